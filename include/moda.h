@@ -381,8 +381,10 @@ moda_status moda_server_create(size_t hbm_budget, void *cuda_stream, moda_server
 moda_status moda_server_submit(moda_server srv, moda_instance inst,
                                const moda_params *params, int64_t *ticket);
 moda_status moda_server_poll(moda_server srv, int64_t ticket, moda_run *done);
-/* Queue state: requests waiting, requests running, bytes of their buffers
- * and the budget (any pointer may be NULL). */
+/* Queue state: requests waiting, requests running (launched and not yet seen
+ * finished: a poll sees its own request's finish, and the server looks at all
+ * of them while a request waits for memory), bytes of their buffers and the
+ * budget (any pointer may be NULL). */
 moda_status moda_server_info(moda_server srv, int64_t *pending, int64_t *running,
                              size_t *bytes_in_use, size_t *budget);
 void moda_server_destroy(moda_server srv);

@@ -6,8 +6,9 @@
  * between the integer thresholds of R21 is accepted when
  *     a <= fl(delta * T[idx]),
  * T[idx] = -ln((idx + 0.5) / 65536) the quantised draw of Sec. 3.1 (R7) and
- * fl the IEEE double product.  The warp engine decides this in FP32 where
- * the FP32 result provably agrees and takes the double test otherwise;
+ * fl the IEEE double product.  The team and the register annealer decide
+ * this in FP32 (one from a float table of T, one from a computed logarithm)
+ * where the FP32 result provably agrees and take the double test otherwise;
  * moda_check_accept runs those same device functions.
  */
 #ifndef MODA_CHECK_H_
@@ -22,8 +23,8 @@ extern "C" {
 #endif
 
 /* For k < count: accept[k] = 1 if a[k] <= fl(delta[k] * T[idx[k]]), else 0,
- * as the device decides it; path[k] = 1 or 0 when the FP32 test decided,
- * -1 when the double test did.  a, delta, idx, accept and path are host
+ * as the device decides it (2 if its two forms of the test differ); path[k] =
+ * 1 or 0 when FP32 decided in both, -1 when a double test did.  a, delta, idx, accept and path are host
  * arrays of `count` entries owned by the caller (accept and path written).
  * Requires a[k] >= 0, delta[k] > 0 and finite, idx[k] < 65536
  * (MODA_EINVAL otherwise, before any device work).  Runs on the current

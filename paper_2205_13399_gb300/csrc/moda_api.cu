@@ -178,6 +178,7 @@ struct moda_instance_s {
   int64_t w1 = 0, w2 = 0;
   int64_t b1 = 0, b2 = 0;  // bounds of the local fields
   int64_t c1max = 0, c2max = 0;  // largest cost-QUBO coefficients
+  int64_t fmax = 0, dmax = 0;    // largest Fs and D entries
   std::vector<int32_t> Fs1, Fs2, D;  // host copies
   int32_t *dFs1 = nullptr, *dFs2 = nullptr, *dD = nullptr;
 };
@@ -209,7 +210,9 @@ struct moda_run_s {
   int32_t *snap_count = nullptr;
   int64_t *snap_E = nullptr;
   uint32_t *snap_bits = nullptr;
-  bool warp = false;  // run by the warp annealer
+  bool warp = false;  // run by the warp or the register annealer
+  bool reg = false;   // the register annealer (moda_reg.cu)
+  uint32_t *arch_min = nullptr;  // its least penalties of slots off chip
   // the warp-annealer launch's shared device buffers (work list, field
   // caches), freed with the last run of that launch
   std::shared_ptr<struct WarpScratch> wscratch;
@@ -266,7 +269,7 @@ cudaError_t free_memory(int dev, size_t *free_b) {
 void free_run_buffers(moda_run r, bool done = false) {
   void *ptrs[] = {r->arch_E, r->arch_bits, r->arch_count, r->x_final,
                   r->E_final, r->stats, r->trace, r->error, r->fcache,
-                  r->snap_count, r->snap_E, r->snap_bits};
+                  r->snap_count, r->snap_E, r->snap_bits, r->arch_min};
   cudaStream_t fs = done ? free_stream(r->inst->device) : r->stream;
   for (void *p : ptrs)
     if (p) cudaFreeAsync(p, fs);
@@ -336,6 +339,53 @@ int warp_slots(moda_instance inst, const moda_params &p) {
 }
 // Archive energies kept in shared memory per warp, at most.
 constexpr int kWarpSmemEnergies = 512;
+
+// Archive slots the register annealer keeps on chip (energies and least
+// penalties), at most: the archives of the workloads reach 528 members.
+constexpr int kRegSlots = 768;
+
+// How a run fits the register annealer at K words per worker: its archive
+// slots on chip (0: it cannot run so) and whether rebuilds use matrix
+// products.  Its packed rows hold 16-bit flows, and everything but the slots
+// must fit in shared memory.
+struct RegFit {
+  int se = 0;
+  bool mma = false;
+};
+RegFit reg_fit(moda_instance inst, int s, int K, bool narrow, int optin) {
+  RegFit f;
+  const int workers = (inst->W + K - 1) / K;
+  if (inst->fmax > 65535 || inst->dmax > 65535 || workers > moda::kRegMaxWorkers) return f;
+  for (const bool mma : {2 * inst->dmax <= 65535, false})
+    for (int se = std::min(s, kRegSlots); se >= 1; se = se > 64 ? se / 2 : se / 8)
+      if ((int64_t)moda::reg_smem(inst->n, inst->m, se, workers, K, !narrow, K >= 4, mma).total <=
+          optin) {
+        f.se = se;
+        f.mma = mma;
+        return f;
+      }
+  return f;
+}
+
+// The words per worker that suit a run best where its launch has the device
+// to itself as far as it can (crowded: no): few words shorten an iteration,
+// and up to n = 35 draw warps take Philox off the workers.
+int reg_words(int W, bool narrow, bool crowded) {
+  if (!crowded) {
+    if (narrow && W <= 20) return 1;
+    if (narrow && W <= 40) return 2;
+    if (W <= 88) return 4;
+    if (W <= 176) return 8;
+  }
+  return W <= 32 ? 4 : W <= 96 ? 8 : W <= 16 * moda::kRegMaxWorkers ? 16 : 24;
+}
+
+// Whether a warp-engine request prescribes the team annealer's layout (team
+// size, prefetch distance, field cache); without that the register
+// annealer, which has none of these, runs it.
+bool prescribes_team(const moda_params *p) {
+  return p->prefetch > 0 || p->block_threads > 0 || p->field_cache == 1 || p->cache_slots > 0;
+}
 
 }  // namespace
 
@@ -415,6 +465,8 @@ moda_status finish_instance(moda_instance inst, const moda_penalty *pen, moda_in
     }
     inst->c1max = e1 * ed;
     inst->c2max = e2 * ed;
+    inst->fmax = std::max(e1, e2);
+    inst->dmax = ed;
   }
   if (b1 >= (int64_t(1) << 31) || b2 >= (int64_t(1) << 31)) {
     delete inst;
@@ -536,6 +588,19 @@ moda_status prepare_warp_run(moda_instance inst, const moda_params *p, cudaStrea
   r->s = p->archive_size > 0 ? p->archive_size : m;
   r->stream = stream;
   r->warp = true;
+  const bool narrow = moda::narrow_ok(inst->n, inst->b1, inst->b2, inst->w1, inst->w2);
+  RegFit fit;
+  if (!prescribes_team(p)) {
+    int optin = 0;
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, inst->device);
+    // the smaller of the slot counts at either choice of words per worker
+    // (the launch is planned later)
+    fit = reg_fit(inst, r->s, reg_words(inst->W, narrow, false), narrow, optin);
+    const RegFit f2 = reg_fit(inst, r->s, reg_words(inst->W, narrow, true), narrow, optin);
+    fit.se = std::min(fit.se, f2.se);
+    fit.mma = fit.mma && f2.mma;
+    r->reg = fit.se > 0;
+  }
   const size_t R = r->R, s = r->s, W = inst->W;
   moda_status st = MODA_OK;
   size_t bytes = 0;
@@ -555,6 +620,7 @@ moda_status prepare_warp_run(moda_instance inst, const moda_params *p, cudaStrea
   alloc((void **)&r->error, sizeof(int32_t));
   if (p->trace && p->I_max > 0)
     alloc((void **)&r->trace, R * (size_t)p->I_max * 3 * sizeof(int64_t));
+  if (r->reg && r->s > fit.se) alloc((void **)&r->arch_min, R * s * sizeof(uint32_t));
   DeviceData *dd = nullptr;
   DeviceData::Sched sch;
   if (st == MODA_OK) {
@@ -577,7 +643,21 @@ moda_status prepare_warp_run(moda_instance inst, const moda_params *p, cudaStrea
   w.m = m;
   w.W = inst->W;
   w.s = r->s;
-  w.narrow = moda::narrow_ok(inst->n, inst->b1, inst->b2, inst->w1, inst->w2) ? 1 : 0;
+  w.narrow = narrow ? 1 : 0;
+  w.se = fit.se;
+  w.mma = fit.mma ? 1 : 0;
+  w.fbig = inst->fmax > 255 ? 1 : 0;
+  w.dmax = (int32_t)std::min<int64_t>(inst->dmax, 65535);
+  w.arch_min = r->arch_min;
+  {
+    // |Delta E_k| <= B_k + w_k (R_i + C_u + 1); the device's largest
+    // R_i + C_u lags by at most three flips (6)
+    int64_t lim = 1 << 20;
+    const int64_t b[2] = {inst->b1, inst->b2}, ww[2] = {inst->w1, inst->w2};
+    for (int k = 0; k < 2; ++k)
+      if (ww[k] > 0) lim = std::min(lim, (INT64_C(2147483646) - b[k]) / ww[k] - 8);
+    w.hm_limit = (int32_t)std::max<int64_t>(lim, -1);
+  }
   w.accept = p->accept;
   w.archive = p->archive;
   w.nsched = sch.count;
@@ -882,14 +962,114 @@ size_t run_bytes(moda_instance inst, const moda_params &p, bool cache) {
   return b;
 }
 
-// A planned launch of the warp annealer.
+// A planned launch of the warp or the register annealer.
 struct WarpGroup {
   std::vector<int> idx;  // its runs
+  bool reg = false;      // register annealer: RL, func, grid, smem
+  moda::RegLaunch RL{};
+  const void *func = nullptr;
+  size_t smem = 0;
   moda::WarpLaunch L{};
   bool narrow = true;
   int grid = 0, warps = 0;
   std::shared_ptr<WarpScratch> scratch;
 };
+
+// Plans one launch of the register annealer over runs[G.idx[k]] (all of one
+// variant and, in a batch, words per worker): allocates and uploads, on
+// `stream`, the run descriptors and the list of replicas (largest runs first,
+// one block each) and clears each run's status word.
+moda_status plan_reg_group(std::vector<moda_run> &runs, std::vector<Prepared> &pls, WarpGroup &G,
+                           cudaStream_t stream) {
+  const moda_run r0 = runs[G.idx[0]];
+  const bool narrow = pls[G.idx[0]].narrow;
+  std::vector<moda::WarpRun> descs;
+  std::vector<std::pair<int, int>> order;  // (-m, k): largest first
+  std::vector<int2> items;
+  int W = 1;
+  for (size_t k = 0; k < G.idx.size(); ++k) {
+    const moda_run r = runs[G.idx[k]];
+    W = std::max(W, r->inst->W);
+    descs.push_back(pls[G.idx[k]].wrun);
+    order.emplace_back(-r->inst->m, (int)k);
+  }
+  std::stable_sort(order.begin(), order.end());
+  for (const auto &o : order)
+    for (int q = 0; q < runs[G.idx[o.second]]->R; ++q) items.push_back(make_int2(o.second, q));
+  int sms = 1, optin = 0;
+  MODA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, r0->inst->device));
+  MODA_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin,
+                                   r0->inst->device));
+  // The fewest words per worker whose blocks are all resident at once, else
+  // the choice for a crowded device.
+  int K = 0, workers = 0, draws = 0;
+  size_t smem = 0;
+  const int crowded = reg_words(W, narrow, true);
+  for (int c = reg_words(W, narrow, false); K == 0; c = c < 8 ? 2 * c : c + 8) {
+    if (c < 4 && crowded < c) continue;
+    const int g = (W + c - 1) / c, d = c < 4 ? (W + 3) / 4 : 0;
+    const bool inl = c >= 4;
+    size_t need = 0;
+    for (const moda::WarpRun &w : descs)
+      need = std::max<size_t>(
+          need, moda::reg_smem(w.n, w.m, w.se, g, c, !narrow, inl, w.mma != 0).total);
+    const void *func = nullptr;
+    int blocks = 0;
+    if (g <= moda::kRegMaxWorkers && (narrow || inl) && need <= (size_t)optin) {
+      cudaError_t e = moda::reg_function(c, narrow, r0->prm.accept != 0, optin, &func);
+      if (e == cudaSuccess) e = moda::reg_occupancy(func, g + d + 2, need, &blocks);
+      if (e != cudaSuccess) {
+        cudaGetLastError();
+        blocks = 0;
+      }
+    }
+    if (blocks >= 1 && ((int64_t)blocks * sms >= (int64_t)items.size() || c >= crowded)) {
+      K = c;
+      workers = g;
+      draws = d;
+      smem = need;
+      G.func = func;
+    } else if (c >= 24) {
+      return fail(MODA_EUNSUPPORTED, "register annealer: the run does not fit a block");
+    }
+  }
+  auto scratch = std::make_shared<WarpScratch>();
+  scratch->device = r0->inst->device;
+  // on failure after this point, work already enqueued may still use the
+  // scratch: wait for the stream before it is freed
+  struct SyncOnFail {
+    cudaStream_t s;
+    bool armed;
+    ~SyncOnFail() {
+      if (armed) cudaStreamSynchronize(s);
+    }
+  } guard{stream, true};
+  const size_t d_bytes = moda::align_up(sizeof(moda::WarpRun) * descs.size(), 256);
+  MODA_CUDA(cudaMallocAsync(&scratch->list, d_bytes + sizeof(int2) * items.size(), stream));
+  unsigned char *base = static_cast<unsigned char *>(scratch->list);
+  MODA_CUDA(cudaMemcpyAsync(base, descs.data(), sizeof(moda::WarpRun) * descs.size(),
+                            cudaMemcpyHostToDevice, stream));
+  MODA_CUDA(cudaMemcpyAsync(base + d_bytes, items.data(), sizeof(int2) * items.size(),
+                            cudaMemcpyHostToDevice, stream));
+  for (int k : G.idx) {
+    moda_run r = runs[k];
+    MODA_CUDA(cudaMemsetAsync(r->error, 0, sizeof(int32_t), stream));
+    r->wscratch = scratch;
+    r->threads = workers;
+    r->bpt = (int)items.size();
+  }
+  G.reg = true;
+  G.narrow = narrow;
+  G.RL.runs = reinterpret_cast<const moda::WarpRun *>(base);
+  G.RL.items = reinterpret_cast<const int2 *>(base + d_bytes);
+  G.RL.workers = workers;
+  G.RL.draws = draws;
+  G.grid = (int)items.size();
+  G.smem = smem;
+  G.scratch = scratch;
+  guard.armed = false;
+  return MODA_OK;
+}
 
 // Plans one launch of the warp annealer over runs[G.idx[k]] (all of one
 // variant, narrow or not): the block shape, the field-cache slots and
@@ -901,6 +1081,7 @@ moda_status plan_warp_group(std::vector<moda_run> &runs, std::vector<Prepared> &
                             WarpGroup &G, cudaStream_t stream, size_t cache_budget) {
   const std::vector<int> &idx = G.idx;
   const moda_run r0 = runs[idx[0]];
+  if (r0->reg) return plan_reg_group(runs, pls, G, stream);
   const int dev = r0->inst->device;
   const bool narrow = pls[idx[0]].narrow;
   int n_max = 2, m_max = 4, s_max = 1, la = 2;
@@ -1160,7 +1341,10 @@ moda_status plan_warp_group(std::vector<moda_run> &runs, std::vector<Prepared> &
 moda_status launch_warp_group(std::vector<moda_run> &runs, const WarpGroup &G,
                               cudaStream_t stream) {
   for (int k : G.idx) MODA_CUDA(cudaEventRecord(runs[k]->start, stream));
-  MODA_CUDA(moda::launch_warp(G.L, G.narrow, G.grid, G.warps, stream));
+  if (G.reg)
+    MODA_CUDA(moda::launch_reg(G.RL, G.func, G.grid, G.smem, stream));
+  else
+    MODA_CUDA(moda::launch_warp(G.L, G.narrow, G.grid, G.warps, stream));
   for (int k : G.idx) MODA_CUDA(cudaEventRecord(runs[k]->stop, stream));
   return MODA_OK;
 }
@@ -1475,14 +1659,23 @@ moda_status moda_anneal_batch(const moda_instance *insts, const moda_params *par
   }
   // Warp-engine runs: one launch per (variant, size class, prefetch
   // distance), a class spanning at most a factor of two in 128-bit chunks
-  // so that no warp's shared memory is sized far beyond its run.
-  std::map<std::tuple<int, int, int>, std::vector<int>> classes;
+  // so that no warp's shared memory is sized far beyond its run; for the
+  // register annealer per (variant, acceptance rule, worker warps), so that
+  // no block has idle warps.
+  std::map<std::tuple<int, int, int, int>, std::vector<int>> classes;
   for (int32_t i = 0; i < count; ++i) {
     if (!runs[i]->warp) continue;
     const int nc = (runs[i]->inst->m + 127) / 128;
+    if (runs[i]->reg) {
+      const int K = reg_words(runs[i]->inst->W, pls[i].narrow, true);
+      classes[std::make_tuple(-K * 100 - (runs[i]->inst->W + K - 1) / K, 1, pls[i].narrow ? 1 : 0,
+                              runs[i]->prm.accept)]
+          .push_back(i);
+      continue;
+    }
     int cls = 0;
     while ((2 << cls) <= nc) ++cls;
-    classes[std::make_tuple(pls[i].narrow ? 1 : 0, -cls, runs[i]->prm.prefetch)].push_back(i);
+    classes[std::make_tuple(pls[i].narrow ? 1 : 0, 0, -cls, runs[i]->prm.prefetch)].push_back(i);
   }
   std::vector<WarpGroup> groups;
   for (auto &kv : classes) {
@@ -1546,16 +1739,19 @@ moda_status moda_anneal_batch(const moda_instance *insts, const moda_params *par
       if (e != cudaSuccess) break;
       starts.push_back(nd);
     }
-    const void *func = nullptr;
-    const size_t smem = (size_t)G.warps * G.L.sm.total;
-    if (e == cudaSuccess) e = moda::warp_function(G.narrow, G.L.nbuf_f > 0, G.L.team, smem, &func);
+    const void *func = G.func;
+    const size_t smem = G.reg ? G.smem : (size_t)G.warps * G.L.sm.total;
+    if (e == cudaSuccess && !G.reg)
+      e = moda::warp_function(G.narrow, G.L.nbuf_f > 0, G.L.team, smem, &func);
     cudaGraphNode_t kn;
     if (e == cudaSuccess) {
-      void *kargs[1] = {const_cast<moda::WarpLaunch *>(&G.L)};
+      void *kargs[1] = {G.reg ? static_cast<void *>(const_cast<moda::RegLaunch *>(&G.RL))
+                              : static_cast<void *>(const_cast<moda::WarpLaunch *>(&G.L))};
       cudaKernelNodeParams kp{};
       kp.func = const_cast<void *>(func);
       kp.gridDim = dim3((unsigned)G.grid);
-      kp.blockDim = dim3((unsigned)(32 * G.warps * G.L.team));
+      kp.blockDim = dim3((unsigned)(G.reg ? 32 * (G.RL.workers + G.RL.draws + 2)
+                                             : 32 * G.warps * G.L.team));
       kp.sharedMemBytes = (unsigned)smem;
       kp.kernelParams = kargs;
       kp.extra = nullptr;
@@ -1625,31 +1821,40 @@ namespace {
 
 constexpr int kServerStreams = 32;
 
-// The server's thread: retires finished runs (their bytes return to the
-// budget) and admits waiting requests in arrival order while their buffers
-// fit the budget, each on a stream of its own, so a request starts as soon
-// as memory allows, beside those already running.
+// Looks whether running request i has finished (caller holds the lock): if
+// so it leaves the list of running ones.
+bool server_retire(moda_server_s *S, size_t i) {
+  auto q = S->running[i];
+  const cudaError_t e = cudaEventQuery(q->run->stop);
+  if (e == cudaErrorNotReady) return false;
+  if (e != cudaSuccess) {
+    q->state = Request::kFailed;
+    q->err = MODA_ECUDA;
+    q->msg = std::string("run: ") + cudaGetErrorString(e);
+  } else {
+    q->state = Request::kDone;
+  }
+  ++S->completed;
+  S->running.erase(S->running.begin() + (long)i);
+  return true;
+}
+
+// The server's thread: admits waiting requests in arrival order while their
+// buffers fit the budget, each on a stream of its own, so a request starts
+// as soon as memory allows, beside those already running.  It sleeps until a
+// request arrives: a run's finish is noticed by its poll (moda_server_poll
+// looks at the run's event itself), and here only while a request waits for
+// memory or the server stops.  (Looking every 100 us instead woke the thread
+// 10,000 times a second under the lock that submit and poll take.)
 void server_loop(moda_server_s *S) {
   cudaSetDevice(S->device);
   std::unique_lock<std::mutex> lock(S->mu);
+  bool blocked = false;  // the first waiting request did not fit
   for (;;) {
-    for (size_t i = 0; i < S->running.size();) {
-      auto &q = S->running[i];
-      const cudaError_t e = cudaEventQuery(q->run->stop);
-      if (e == cudaErrorNotReady) {
-        ++i;
-        continue;
-      }
-      if (e != cudaSuccess) {
-        q->state = Request::kFailed;
-        q->err = MODA_ECUDA;
-        q->msg = std::string("run: ") + cudaGetErrorString(e);
-      } else {
-        q->state = Request::kDone;
-      }
-      ++S->completed;
-      S->running.erase(S->running.begin() + (long)i);
-    }
+    if (blocked || S->stopping)
+      for (size_t i = 0; i < S->running.size();)
+        if (!server_retire(S, i)) ++i;
+    blocked = false;
     while (!S->pending.empty()) {
       std::shared_ptr<Request> q = S->pending.front();
       if (S->stopping) {  // not started: cancelled
@@ -1664,9 +1869,15 @@ void server_loop(moda_server_s *S) {
       const size_t lean = run_bytes(q->inst, prm, false);
       const size_t in_use = S->acct->in_use.load();
       if (in_use + full > S->budget) {
-        if (!S->running.empty()) break;  // wait for memory
+        if (!S->running.empty()) {  // wait for memory
+          blocked = true;
+          break;
+        }
         if (in_use + lean > S->budget) {
-          if (in_use > 0) break;  // wait for the caller's runs to be destroyed
+          if (in_use > 0) {  // wait for the caller's runs to be destroyed
+            blocked = true;
+            break;
+          }
           q->state = Request::kFailed;
           q->err = MODA_ENOMEM;
           q->msg = "request needs " + std::to_string(lean) + " bytes, budget " +
@@ -1707,6 +1918,7 @@ void server_loop(moda_server_s *S) {
       }
       if (rs == MODA_ENOMEM && (!S->running.empty() || S->acct->in_use.load() > 0)) {
         S->pending.push_front(q);  // memory held elsewhere: retry when it frees
+        blocked = true;
         break;
       }
       if (rs != MODA_OK) {
@@ -1724,7 +1936,10 @@ void server_loop(moda_server_s *S) {
       S->running.push_back(q);
     }
     if (S->stopping && S->pending.empty() && S->running.empty()) break;
-    S->cv.wait_for(lock, std::chrono::microseconds(S->running.empty() ? 2000 : 100));
+    if (blocked || S->stopping)
+      S->cv.wait_for(lock, std::chrono::microseconds(100));
+    else
+      S->cv.wait(lock, [&] { return S->stopping || !S->pending.empty(); });
   }
 }
 
@@ -1799,6 +2014,12 @@ moda_status moda_server_poll(moda_server S, int64_t ticket, moda_run *done) {
   auto it = S->tickets.find(ticket);
   if (it == S->tickets.end()) return fail(MODA_EINVAL, "unknown ticket");
   std::shared_ptr<Request> q = it->second;
+  if (q->state == Request::kRunning)
+    for (size_t i = 0; i < S->running.size(); ++i)
+      if (S->running[i] == q) {
+        server_retire(S, i);
+        break;
+      }
   if (q->state == Request::kDone) {
     *done = q->run;
     S->tickets.erase(it);
@@ -1989,7 +2210,10 @@ moda_status moda_autotune(moda_instance inst, const moda_params *params, int32_t
     bool found = false;
     float fastest = 0.f;
     moda_params winner = *params;
-    for (int32_t pf : {1, 3, 7, 11, 15}) {
+    // (0, the register annealer, first where the engine is left open; a
+    // request for the warp engine gets one of its team annealer's layouts)
+    for (int32_t pf : {0, 1, 3, 7, 11, 15}) {
+      if (pf == 0 && (params->engine != 0 || prescribes_team(params))) continue;
       trial.prefetch = pf;
       moda_run r = nullptr;
       if (moda_anneal(inst, &trial, stream, &r) != MODA_OK) continue;

@@ -194,6 +194,29 @@ __device__ __forceinline__ int prefilter(float af, float df, float Tf) {
   return -1;
 }
 
+// The same test with -ln u computed instead of loaded (a gather from a
+// 256 KB table misses L1 on most lanes): with v = idx + 0.5 (exact in
+// float), delta T = delta ln 2 (16 - log2 v).  accept_level is that up to:
+// lg2.approx's error (at most 2^-22.6 relative or absolute, so 2.6e-6 of
+// log2 v <= 16, 1.8e-6 delta) and the rounding of fl32(delta ln 2) and of
+// the fused difference (2^-24 each, of at most 11.8 delta).  With the
+// rounding of fl32(a) and of a - level (2^-24 each, of at most 11.8 delta
+// where they are close) the difference is within 6e-6 delta of a - delta T;
+// the caller hands |a - level| <= accept_margin = 2e-5 delta to the double
+// test.
+__device__ __forceinline__ float accept_scale(double delta) {
+  return (float)(delta * 0.69314718055994530942);
+}
+__device__ __forceinline__ float accept_margin(double delta) { return (float)delta * 2e-5f; }
+// fl32(delta T) of a draw, cln = accept_scale(delta)
+__device__ __forceinline__ float accept_level(uint32_t word, float cln) {
+  // top 16 bits of the word as a float: 2^23 + idx, less 2^23 - 0.5
+  const float v = __uint_as_float(__byte_perm(word, 0x4B00u, 0x5432u)) - 8388607.5f;
+  float lg;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(v));
+  return __fmaf_rn(-lg, cln, 16.f * cln);
+}
+
 // Inclusive prefix sum of `v` over the lanes.
 __device__ __forceinline__ int warp_incl_scan(int v, int lane) {
 #pragma unroll

@@ -364,6 +364,12 @@ struct WarpRun {
   int64_t *stats;
   int64_t *trace;            // [R][I_max][3] or nullptr
   int32_t *error;
+  // register annealer (moda_reg.cu): least penalties of archive slots >= se
+  // [R][s] or nullptr; largest R_i + C_u at which every Delta E fits int32
+  uint32_t *arch_min;
+  int32_t hm_limit;
+  int32_t mma;               // rebuilds by matrix products: 2 max d < 2^16 and room
+  int32_t fbig, dmax;        // some Fs entry > 255; largest distance
 };
 
 // Kernel argument of a warp-annealer launch.
@@ -408,6 +414,86 @@ cudaError_t launch_check_accept(const int64_t *a, const double *delta, const uin
                                 int8_t *path, cudaStream_t stream);
 // Resident blocks (one team of `team` warps each) per SM of that variant.
 cudaError_t warp_occupancy(bool narrow, bool fz, int team, size_t smem, int *blocks);
+
+// ---- the register annealer: one block per replica, Delta E in registers ----
+//
+// Worker warps own K state words each, draw warps (if any) prepare the
+// acceptance draws, a scan and a store warp keep the archive; see
+// moda_reg_body.cuh.
+
+// Outcome of a round of jumps, told to the block: the run ends on an archive
+// member, goes on from one, stays at its state (empty archive), or ends there.
+enum : uint32_t { kRegEnd = 0, kRegRebuild = 1, kRegStay = 2, kRegStayEnd = 3 };
+
+constexpr int kRegRing = 128;      // schedule / draw ring entries (iterations)
+constexpr int kRegMaxWorkers = 26;
+
+// Flow pairs as two int32 (fewer instructions) where they are small.
+__host__ __device__ constexpr bool reg_f64(int K) { return K <= 8; }
+// Registers per thread: what K words of Delta E need without spilling in the
+// flip's round, and as many resident blocks as that leaves.
+__host__ __device__ constexpr int reg_regs(int K) {
+  return K <= 4 ? 64 : K == 8 ? 80 : K == 16 ? 72 : 96;
+}
+
+// Rebuild by matrix products (flag mma of a run): M^T as bytes, one row per
+// column u (padded to tiles of 8), `mstride` bytes a row (k padded to 32,
+// plus 16 so that the eight rows of a fragment fall in different banks).
+__host__ __device__ inline int reg_mstride(int n) { return (n + 31) / 32 * 32 + 16; }
+
+struct RegSmem {
+  uint32_t fs, d, ring, cnt, min, flip, tgt, jump, rc, v2, x, sum, rcp, draw, scr, mt, aE, aM,
+      total;
+};
+__host__ __device__ inline RegSmem reg_smem(int n, int m, int se, int workers, int K, bool wide,
+                                            bool inl, bool mma) {
+  const int nc = (m + 127) / 128;
+  RegSmem L;
+  size_t o = 0;
+  L.fs = 0;              o = align_up((size_t)(reg_f64(K) ? 8 : 4) * n * (n + 1), 16);
+  L.d = (uint32_t)o;     o = align_up(o + 4 * (size_t)m, 16);
+  L.ring = (uint32_t)o;  o = align_up(o + 32 * (size_t)kRegRing, 16);
+  L.cnt = (uint32_t)o;   o = align_up(o + 4 * 2 * 32, 16);
+  L.min = (uint32_t)o;   o = align_up(o + 4 * 2 * 32, 16);
+  L.flip = (uint32_t)o;  o = align_up(o + 4 * 32, 16);
+  L.tgt = (uint32_t)o;   o = align_up(o + 4 * 4, 16);
+  L.jump = (uint32_t)o;  o = align_up(o + 32, 16);
+  L.rc = (uint32_t)o;    o = align_up(o + 4 * 2 * (size_t)kMaxN, 16);
+  L.v2 = (uint32_t)o;    o = align_up(o + 2 * (size_t)kMaxN, 16);
+  L.x = (uint32_t)o;     o = align_up(o + 16 * (size_t)nc, 16);
+  L.sum = (uint32_t)o;   o = align_up(o + 16 * 32, 16);
+  L.rcp = (uint32_t)o;   if (wide) o = align_up(o + 2 * (size_t)kMaxN * (size_t)workers, 16);
+  // levels: of two iterations, or of one chunk per worker
+  L.draw = (uint32_t)o;  o = align_up(o + 512 * (inl ? (size_t)workers : 2 * (size_t)nc), 16);
+  // a strip of 16 rows of (L_1, L_2), or 32 rows of M = X D
+  L.scr = (uint32_t)o;   o = align_up(o + 8 * 16 * (size_t)n, 16);
+  L.mt = (uint32_t)o;
+  if (mma) o = align_up(o + 2 * (size_t)((n + 7) / 8 * 8) * reg_mstride(n), 16);
+  // archive slots on chip, and one that only takes stores
+  L.aE = (uint32_t)o;    o = align_up(o + 16 * ((size_t)se + 1), 16);
+  L.aM = (uint32_t)o;    o = align_up(o + 4 * ((size_t)se + 1), 16);
+  L.total = (uint32_t)o;
+  return L;
+}
+
+struct RegLaunch {
+  const WarpRun *runs;
+  const int2 *items;  // (run, replica row), one block each, largest runs first
+  int32_t workers;    // G
+  int32_t draws;      // D (0 with inline draws)
+};
+
+// The kernel with K words per worker (1, 2 with draw warps and int32 Delta E
+// only; 4, 8, 16, 24 with inline draws), with `optin` bytes of dynamic shared
+// memory allowed, its resident blocks per SM and its launch.
+cudaError_t reg_function(int K, bool narrow, bool lenient, int optin, const void **func);
+const void *reg_kernel_strict(int K, bool narrow);
+const void *reg_kernel_lenient(int K, bool narrow);
+const void *reg_kernel_strict_wide(int K);
+const void *reg_kernel_lenient_wide(int K);
+cudaError_t reg_occupancy(const void *func, int warps, size_t smem, int *blocks);
+cudaError_t launch_reg(const RegLaunch &L, const void *func, int grid, size_t smem,
+                       cudaStream_t stream);
 
 // Sets the thread-local message that moda_last_error() returns.
 void set_last_error(const char *msg);

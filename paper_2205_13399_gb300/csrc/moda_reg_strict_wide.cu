@@ -1,0 +1,15 @@
+// Register annealer, strict acceptance, Delta E beyond int32 (see
+// moda_reg_body.cuh).
+#include "moda_reg_body.cuh"
+
+namespace moda {
+
+const void *reg_kernel_strict_wide(int K) {
+  return K == 4    ? reinterpret_cast<const void *>(reg_anneal_kernel<4, true, false, true>)
+         : K == 8  ? reinterpret_cast<const void *>(reg_anneal_kernel<8, true, false, true>)
+         : K == 16 ? reinterpret_cast<const void *>(reg_anneal_kernel<16, true, false, true>)
+         : K == 24 ? reinterpret_cast<const void *>(reg_anneal_kernel<24, true, false, true>)
+                   : nullptr;
+}
+
+}  // namespace moda

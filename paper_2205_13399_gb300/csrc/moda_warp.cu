@@ -1436,9 +1436,10 @@ __global__ void __launch_bounds__(256, 1) warp_anneal_kernel(const WarpLaunch L)
 }  // namespace
 
 namespace {
-// The warp engine's acceptance decision for given penalties, one per thread
-// (the same device functions its trials run): accept[k] and the path taken
-// (1 or 0 decided in FP32, -1 by the double test).
+// The acceptance decisions of the team annealer (prefilter) and of the
+// register annealer (accept_level) for given penalties, one per thread (the
+// same device functions their trials run): accept[k], 2 if they differ, and
+// the path taken (1 or 0 decided in FP32 by both, -1 by the double test).
 __global__ void check_accept_kernel(const int64_t *a, const double *delta, const uint32_t *idx,
                                     int count, const double *T, const float *Tf,
                                     uint8_t *accept, int8_t *path) {
@@ -1448,8 +1449,13 @@ __global__ void check_accept_kernel(const int64_t *a, const double *delta, const
   const double dk = delta[k];
   const uint32_t ik = idx[k];
   const int r = prefilter(penalty_f32(ak), __double2float_rn(dk), Tf[ik]);
-  accept[k] = (uint8_t)(r > 0 || (r < 0 && (double)ak <= __dmul_rn(dk, T[ik])));
-  path[k] = (int8_t)r;
+  const bool exact = (double)ak <= __dmul_rn(dk, T[ik]);
+  const bool team = r > 0 || (r < 0 && exact);
+  const float diff = penalty_f32(ak) - accept_level(ik << 16, accept_scale(dk));
+  const bool near = fabsf(diff) <= accept_margin(dk);
+  const bool reg = near ? exact : diff < 0.f;
+  accept[k] = team == reg ? (uint8_t)team : (uint8_t)2;
+  path[k] = near ? (int8_t)-1 : (int8_t)r;
 }
 
 // The kernel variant of a launch: narrow or not.
