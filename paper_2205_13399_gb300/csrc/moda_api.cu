@@ -1480,24 +1480,41 @@ moda_status archive_front(moda_run r, int32_t rep, moda_point *pts, int32_t cap,
                           int32_t *count, uint8_t *perms, const int32_t *dcnt,
                           const int64_t *dE, const uint32_t *dbits, size_t ns, size_t j) {
   const int n = r->inst->n, W = r->inst->W;
-  const size_t s = r->s;
+  const int s = r->s;
   const int first = rep < 0 ? 0 : rep, last = rep < 0 ? r->R : rep + 1;
-  struct Cand {
-    int64_t e1, e2;
-    int32_t rep, slot;
-  };
-  std::vector<Cand> c;
-  std::vector<int64_t> E(s * 2);
-  for (int q = first; q < last; ++q) {
-    int32_t cnt = 0;
-    const size_t row = (size_t)q * ns + j;
-    MODA_CUDA(cudaMemcpy(&cnt, dcnt + row, sizeof(int32_t), cudaMemcpyDeviceToHost));
-    if (cnt <= 0) continue;
-    MODA_CUDA(cudaMemcpy(E.data(), dE + row * s * 2, sizeof(int64_t) * 2 * (size_t)cnt,
-                         cudaMemcpyDeviceToHost));
-    for (int32_t k = 0; k < cnt; ++k) c.push_back({E[2 * k], E[2 * k + 1], q, k});
+  // the archive sizes bound the packed list
+  cudaStream_t st = free_stream(r->inst->device);
+  std::vector<int32_t> cnt((size_t)(last - first));
+  MODA_CUDA(cudaMemcpy2DAsync(cnt.data(), sizeof(int32_t), dcnt + (size_t)first * ns + j,
+                              sizeof(int32_t) * ns, sizeof(int32_t), cnt.size(),
+                              cudaMemcpyDeviceToHost, st));
+  MODA_CUDA(cudaStreamSynchronize(st));
+  size_t most = 0;
+  for (int32_t q : cnt) most += (size_t)std::min(std::max(q, 0), s);
+  struct Buffer {  // device scratch, given back in stream order
+    cudaStream_t st;
+    void *p = nullptr;
+    ~Buffer() {
+      if (p) cudaFreeAsync(p, st);
+    }
+  } list{st}, words{st};
+  std::vector<moda::FrontPoint> c;
+  if (most > 0) {
+    const size_t head = 16;
+    MODA_CUDA(cudaMallocAsync(&list.p, head + most * sizeof(moda::FrontPoint), st));
+    auto *total = static_cast<uint32_t *>(list.p);
+    auto *out = reinterpret_cast<moda::FrontPoint *>(static_cast<unsigned char *>(list.p) + head);
+    MODA_CUDA(cudaMemsetAsync(total, 0, sizeof(uint32_t), st));
+    MODA_CUDA(moda::launch_front(dcnt, dE, s, (int)ns, (int)j, first, last - first, out, total, st));
+    uint32_t got = 0;
+    MODA_CUDA(cudaMemcpyAsync(&got, total, sizeof(got), cudaMemcpyDeviceToHost, st));
+    MODA_CUDA(cudaStreamSynchronize(st));
+    c.resize(got);
+    MODA_CUDA(cudaMemcpyAsync(c.data(), out, sizeof(moda::FrontPoint) * got,
+                              cudaMemcpyDeviceToHost, st));
+    MODA_CUDA(cudaStreamSynchronize(st));
   }
-  std::sort(c.begin(), c.end(), [](const Cand &a, const Cand &b) {
+  std::sort(c.begin(), c.end(), [](const moda::FrontPoint &a, const moda::FrontPoint &b) {
     if (a.e1 != b.e1) return a.e1 < b.e1;
     if (a.e2 != b.e2) return a.e2 < b.e2;
     if (a.rep != b.rep) return a.rep < b.rep;
@@ -1506,10 +1523,10 @@ moda_status archive_front(moda_run r, int32_t rep, moda_point *pts, int32_t cap,
   // Sweep in E1 order: a point survives iff its E2 is below every E2 seen
   // so far (points with equal E1 and larger E2 are dominated; equal vectors
   // keep the first, i.e. the lowest (replica, slot)).
-  std::vector<Cand> keep;
+  std::vector<moda::FrontPoint> keep;
   bool any = false;
   int64_t best2 = 0;
-  for (const Cand &q : c) {
+  for (const moda::FrontPoint &q : c) {
     if (!any || q.e2 < best2) {
       keep.push_back(q);
       best2 = q.e2;
@@ -1518,11 +1535,23 @@ moda_status archive_front(moda_run r, int32_t rep, moda_point *pts, int32_t cap,
   }
   *count = (int32_t)keep.size();
   const int wr = std::min<int32_t>(cap, (int32_t)keep.size());
-  std::vector<uint32_t> word(W);
+  // their states, in one copy
+  std::vector<uint32_t> state((size_t)wr * W);
+  if (wr > 0) {
+    const size_t pb = moda::align_up(sizeof(moda::FrontPoint) * (size_t)wr, 16);
+    MODA_CUDA(cudaMallocAsync(&words.p, pb + sizeof(uint32_t) * state.size(), st));
+    auto *pts_d = static_cast<moda::FrontPoint *>(words.p);
+    auto *out = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(words.p) + pb);
+    MODA_CUDA(cudaMemcpyAsync(pts_d, keep.data(), sizeof(moda::FrontPoint) * (size_t)wr,
+                              cudaMemcpyHostToDevice, st));
+    MODA_CUDA(moda::launch_gather(dbits, pts_d, wr, s, (int)ns, (int)j, W, out, st));
+    MODA_CUDA(cudaMemcpyAsync(state.data(), out, sizeof(uint32_t) * state.size(),
+                              cudaMemcpyDeviceToHost, st));
+    MODA_CUDA(cudaStreamSynchronize(st));
+  }
   for (int k = 0; k < wr; ++k) {
-    const Cand &q = keep[k];
-    MODA_CUDA(cudaMemcpy(word.data(), dbits + (((size_t)q.rep * ns + j) * s + q.slot) * W,
-                         W * sizeof(uint32_t), cudaMemcpyDeviceToHost));
+    const moda::FrontPoint &q = keep[k];
+    const uint32_t *word = state.data() + (size_t)k * W;
     std::vector<int> rows(n, 0), cols(n, 0), loc(n, -1);
     for (int p = 0; p < n * n; ++p)
       if ((word[p >> 5] >> (p & 31)) & 1u) {

@@ -495,6 +495,22 @@ cudaError_t reg_occupancy(const void *func, int warps, size_t smem, int *blocks)
 cudaError_t launch_reg(const RegLaunch &L, const void *func, int grid, size_t smem,
                        cudaStream_t stream);
 
+// ---- fronts (moda_front.cu) -------------------------------------------------
+
+// A member of an archive: its energies, replica and slot.
+struct FrontPoint {
+  int64_t e1, e2;
+  int32_t rep, slot;
+};
+// The non-dominated members of each of the archives of replicas first ..
+// first + rows - 1 (counts[q * ns + j], energies E + (q * ns + j) * s * 2),
+// packed in no order into out; *total must be 0 before.
+cudaError_t launch_front(const int32_t *counts, const int64_t *E, int s, int ns, int j, int first,
+                         int rows, FrontPoint *out, uint32_t *total, cudaStream_t stream);
+// The states (W words each) of n members.
+cudaError_t launch_gather(const uint32_t *bits, const FrontPoint *pts, int n, int s, int ns, int j,
+                          int W, uint32_t *out, cudaStream_t stream);
+
 // Sets the thread-local message that moda_last_error() returns.
 void set_last_error(const char *msg);
 inline void set_last_error(const std::string &msg) { set_last_error(msg.c_str()); }

@@ -87,6 +87,10 @@ class Point(ctypes.Structure):
     ]
 
 
+_POINT = np.dtype([(k, np.int64) for k in ("E1", "E2", "c1", "c2", "g")]
+                  + [(k, np.int32) for k in ("feasible", "replica", "slot", "pad")])
+
+
 class DeviceOutputs(ctypes.Structure):
     """Device output buffers of moda_anneal_noalloc (caller-owned)."""
     _fields_ = [
@@ -331,13 +335,14 @@ class Run:
         pts = (Point * max(total, 1))()
         pbuf = np.zeros((max(total, 1), self.inst.n), dtype=np.uint8)
         _check(call(pts, total, ctypes.byref(cnt), _ptr(pbuf) if perms else None))
+        rows = np.frombuffer(pts, dtype=_POINT)[:total].tolist()  # plain ints, field order
+        pl = pbuf.tolist() if perms else None
         out = []
-        for k in range(total):
-            p = pts[k]
-            d = dict(E1=p.E1, E2=p.E2, c1=p.c1, c2=p.c2, g=p.g, feasible=bool(p.feasible),
-                     replica=p.replica, slot=p.slot)
+        for k, (E1, E2, c1, c2, g, feasible, rep, slot, _) in enumerate(rows):
+            d = dict(E1=E1, E2=E2, c1=c1, c2=c2, g=g, feasible=bool(feasible), replica=rep,
+                     slot=slot)
             if perms:
-                d["perm"] = [int(v) for v in pbuf[k]] if p.feasible else None
+                d["perm"] = pl[k] if feasible else None
             out.append(d)
         return out
 
