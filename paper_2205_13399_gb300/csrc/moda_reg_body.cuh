@@ -1056,6 +1056,23 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     bool end = false;
     const uint32_t ring_to = t + 46u;  // the ring holds the iterations up to here
     for (;;) {
+      if (trace == nullptr && t >= nsched) {
+        // the schedule is frozen: four batches' draws at a time (they hide
+        // one another's latency) while no member may accept
+        while (I_max - t >= 128u) {
+          bool live = false;
+#pragma unroll
+          for (uint32_t g = 0; g < 4u; ++g) {
+            uint32_t d[4] = {0u, t + 32u * g + (uint32_t)lane, rep, kTagRestart};
+            philox10(d, k0, k1);
+            const int y = pick(d[0], acount);
+            live |= (y < se ? sAM[y] : gM[y]) <= hiF32;
+          }
+          if (__any_sync(kFull, live)) break;
+          njump += 128u;
+          t += 128u;
+        }
+      }
       const uint32_t it = t + (uint32_t)lane;  // may pass I_max: such lanes stop
       uint32_t d[4] = {0u, it, rep, kTagRestart};
       philox10(d, k0, k1);
