@@ -310,6 +310,13 @@ bool warp_options(const moda_params *p) {
          p->fast_forward == 0;
 }
 
+// Whether a request runs on the block engine unless the register annealer
+// can take it: the engine left open, with an option of the extensions.
+bool reg_extension(const moda_params *p) {
+  return p->engine == 0 && !warp_options(p) && p->fast_forward == 0 && p->block_threads == 0 &&
+         p->prefetch == 0 && p->field_cache != 1 && p->cache_slots == 0;
+}
+
 // Whether prepare_run gives a request to the warp annealer.
 bool uses_warp(const moda_params *p) {
   return p->engine == 2 || (p->engine == 0 && warp_options(p) && p->block_threads == 0);
@@ -352,13 +359,13 @@ struct RegFit {
   int se = 0;
   bool mma = false;
 };
-RegFit reg_fit(moda_instance inst, int s, int K, bool narrow, int optin) {
+RegFit reg_fit(moda_instance inst, int s, int K, bool wide, int optin) {
   RegFit f;
   const int workers = (inst->W + K - 1) / K;
   if (inst->fmax > 65535 || inst->dmax > 65535 || workers > moda::kRegMaxWorkers) return f;
   for (const bool mma : {2 * inst->dmax <= 65535, false})
     for (int se = std::min(s, kRegSlots); se >= 1; se = se > 64 ? se / 2 : se / 8)
-      if ((int64_t)moda::reg_smem(inst->n, inst->m, se, workers, K, !narrow, K >= 4, mma).total <=
+      if ((int64_t)moda::reg_smem(inst->n, inst->m, se, workers, K, wide, K >= 4, mma).total <=
           optin) {
         f.se = se;
         f.mma = mma;
@@ -369,15 +376,31 @@ RegFit reg_fit(moda_instance inst, int s, int K, bool narrow, int optin) {
 
 // The words per worker that suit a run best where its launch has the device
 // to itself as far as it can (crowded: no): few words shorten an iteration,
-// and up to n = 35 draw warps take Philox off the workers.
-int reg_words(int W, bool narrow, bool crowded) {
+// and up to n = 35 draw warps take Philox off the workers (draws: the kernel
+// has such variants).
+int reg_words(int W, bool draws, bool crowded) {
   if (!crowded) {
-    if (narrow && W <= 20) return 1;
-    if (narrow && W <= 40) return 2;
+    if (draws && W <= 20) return 1;
+    if (draws && W <= 40) return 2;
     if (W <= 88) return 4;
     if (W <= 176) return 8;
   }
   return W <= 32 ? 4 : W <= 96 ? 8 : W <= 16 * moda::kRegMaxWorkers ? 16 : 24;
+}
+
+// reg_fit at either choice of words per worker (the launch is planned
+// later): the smaller of the slot counts.
+RegFit reg_plan(moda_instance inst, const moda_params *p, bool narrow) {
+  int optin = 0;
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, inst->device);
+  const bool ext = !warp_options(p);
+  const int s = p->archive_size > 0 ? p->archive_size : inst->m;
+  const bool draws = narrow || ext, wide = !narrow || ext;
+  RegFit f = reg_fit(inst, s, reg_words(inst->W, draws, false), wide, optin);
+  const RegFit g = reg_fit(inst, s, reg_words(inst->W, draws, true), wide, optin);
+  f.se = std::min(f.se, g.se);
+  f.mma = f.mma && g.mma;
+  return f;
 }
 
 // Whether a warp-engine request prescribes the team annealer's layout (team
@@ -590,17 +613,8 @@ moda_status prepare_warp_run(moda_instance inst, const moda_params *p, cudaStrea
   r->warp = true;
   const bool narrow = moda::narrow_ok(inst->n, inst->b1, inst->b2, inst->w1, inst->w2);
   RegFit fit;
-  if (!prescribes_team(p)) {
-    int optin = 0;
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, inst->device);
-    // the smaller of the slot counts at either choice of words per worker
-    // (the launch is planned later)
-    fit = reg_fit(inst, r->s, reg_words(inst->W, narrow, false), narrow, optin);
-    const RegFit f2 = reg_fit(inst, r->s, reg_words(inst->W, narrow, true), narrow, optin);
-    fit.se = std::min(fit.se, f2.se);
-    fit.mma = fit.mma && f2.mma;
-    r->reg = fit.se > 0;
-  }
+  if (!prescribes_team(p)) fit = reg_plan(inst, p, narrow);
+  r->reg = fit.se > 0;
   const size_t R = r->R, s = r->s, W = inst->W;
   moda_status st = MODA_OK;
   size_t bytes = 0;
@@ -620,6 +634,15 @@ moda_status prepare_warp_run(moda_instance inst, const moda_params *p, cudaStrea
   alloc((void **)&r->error, sizeof(int32_t));
   if (p->trace && p->I_max > 0)
     alloc((void **)&r->trace, R * (size_t)p->I_max * 3 * sizeof(int64_t));
+  if (p->snapshot_every > 0) {  // as many as fit the run (register annealer only)
+    r->nsnap = (int32_t)(p->I_max / p->snapshot_every);
+    const size_t ns = (size_t)r->nsnap;
+    if (ns > 0) {
+      alloc((void **)&r->snap_count, R * ns * sizeof(int32_t));
+      alloc((void **)&r->snap_E, R * ns * s * 2 * sizeof(int64_t));
+      alloc((void **)&r->snap_bits, R * ns * s * W * sizeof(uint32_t));
+    }
+  }
   if (r->reg && r->s > fit.se) alloc((void **)&r->arch_min, R * s * sizeof(uint32_t));
   DeviceData *dd = nullptr;
   DeviceData::Sched sch;
@@ -658,6 +681,16 @@ moda_status prepare_warp_run(moda_instance inst, const moda_params *p, cudaStrea
       if (ww[k] > 0) lim = std::min(lim, (INT64_C(2147483646) - b[k]) / ww[k] - 8);
     w.hm_limit = (int32_t)std::max<int64_t>(lim, -1);
   }
+  w.normalize = p->normalize;
+  w.escape = p->escape;
+  w.beta = p->beta;
+  w.s1 = p->normalize ? moda::norm_scale(inst->c1max) : 1.0;
+  w.s2 = p->normalize ? moda::norm_scale(inst->c2max) : 1.0;
+  w.snap_every = p->snapshot_every;
+  w.nsnap = r->nsnap;
+  w.snap_count = r->snap_count;
+  w.snap_E = r->snap_E;
+  w.snap_bits = r->snap_bits;
   w.accept = p->accept;
   w.archive = p->archive;
   w.nsched = sch.count;
@@ -726,6 +759,12 @@ moda_status prepare_run(moda_instance inst, const moda_params *p,
                 "the warp engine needs the archive escape without normalize, "
                 "snapshot_every or fast_forward");
   if (uses_warp(p)) return prepare_warp_run(inst, p, stream, out, pl);
+  // (checked here as the block engine checks them below)
+  if (reg_extension(p) && p->field_cache >= 0 && p->field_cache <= 2 &&
+      (p->normalize == 0 || p->normalize == 1) && p->snapshot_every >= 0 &&
+      (p->snapshot_every == 0 || p->I_max / p->snapshot_every <= 1000000) &&
+      reg_plan(inst, p, moda::narrow_ok(inst->n, inst->b1, inst->b2, inst->w1, inst->w2)).se > 0)
+    return prepare_warp_run(inst, p, stream, out, pl);
 
   // Block shape: B rounds of T threads own the bits, B * T >= m.
   static const int kRounds[] = {1, 2, 3, 4, 6, 8};
@@ -1004,19 +1043,20 @@ moda_status plan_reg_group(std::vector<moda_run> &runs, std::vector<Prepared> &p
   // the choice for a crowded device.
   int K = 0, workers = 0, draws = 0;
   size_t smem = 0;
-  const int crowded = reg_words(W, narrow, true);
-  for (int c = reg_words(W, narrow, false); K == 0; c = c < 8 ? 2 * c : c + 8) {
+  const bool ext = !warp_options(&r0->prm), wide = !narrow || ext, draw_warps = narrow || ext;
+  const int crowded = reg_words(W, draw_warps, true);
+  for (int c = reg_words(W, draw_warps, false); K == 0; c = c < 8 ? 2 * c : c + 8) {
     if (c < 4 && crowded < c) continue;
     const int g = (W + c - 1) / c, d = c < 4 ? (W + 3) / 4 : 0;
     const bool inl = c >= 4;
     size_t need = 0;
     for (const moda::WarpRun &w : descs)
       need = std::max<size_t>(
-          need, moda::reg_smem(w.n, w.m, w.se, g, c, !narrow, inl, w.mma != 0).total);
+          need, moda::reg_smem(w.n, w.m, w.se, g, c, wide, inl, w.mma != 0).total);
     const void *func = nullptr;
     int blocks = 0;
-    if (g <= moda::kRegMaxWorkers && (narrow || inl) && need <= (size_t)optin) {
-      cudaError_t e = moda::reg_function(c, narrow, r0->prm.accept != 0, optin, &func);
+    if (g <= moda::kRegMaxWorkers && (draw_warps || inl) && need <= (size_t)optin) {
+      cudaError_t e = moda::reg_function(c, narrow, r0->prm.accept != 0, ext, optin, &func);
       if (e == cudaSuccess) e = moda::reg_occupancy(func, g + d + 2, need, &blocks);
       if (e != cudaSuccess) {
         cudaGetLastError();
@@ -1696,9 +1736,10 @@ moda_status moda_anneal_batch(const moda_instance *insts, const moda_params *par
     if (!runs[i]->warp) continue;
     const int nc = (runs[i]->inst->m + 127) / 128;
     if (runs[i]->reg) {
-      const int K = reg_words(runs[i]->inst->W, pls[i].narrow, true);
-      classes[std::make_tuple(-K * 100 - (runs[i]->inst->W + K - 1) / K, 1, pls[i].narrow ? 1 : 0,
-                              runs[i]->prm.accept)]
+      const int K = reg_words(runs[i]->inst->W, true, true);
+      const bool ext = !warp_options(&runs[i]->prm);
+      classes[std::make_tuple(-K * 100 - (runs[i]->inst->W + K - 1) / K, 1,
+                              ext ? 2 : pls[i].narrow ? 1 : 0, ext ? 0 : runs[i]->prm.accept)]
           .push_back(i);
       continue;
     }

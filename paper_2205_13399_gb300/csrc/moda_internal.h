@@ -370,6 +370,14 @@ struct WarpRun {
   int32_t hm_limit;
   int32_t mma;               // rebuilds by matrix products: 2 max d < 2^16 and room
   int32_t fbig, dmax;        // some Fs entry > 255; largest distance
+  // its extensions (ext of the launch): normalisation with its scales, the
+  // offset escape, archive snapshots (moda_params)
+  int32_t normalize, escape, snap_every, nsnap;
+  double s1, s2;
+  int64_t beta;
+  int32_t *snap_count;       // [R][nsnap]
+  int64_t *snap_E;           // [R][nsnap][s][2]
+  uint32_t *snap_bits;       // [R][nsnap][s][W]
 };
 
 // Kernel argument of a warp-annealer launch.
@@ -486,11 +494,13 @@ struct RegLaunch {
 // The kernel with K words per worker (1, 2 with draw warps and int32 Delta E
 // only; 4, 8, 16, 24 with inline draws), with `optin` bytes of dynamic shared
 // memory allowed, its resident blocks per SM and its launch.
-cudaError_t reg_function(int K, bool narrow, bool lenient, int optin, const void **func);
+cudaError_t reg_function(int K, bool narrow, bool lenient, bool ext, int optin,
+                         const void **func);
 const void *reg_kernel_strict(int K, bool narrow);
 const void *reg_kernel_lenient(int K, bool narrow);
 const void *reg_kernel_strict_wide(int K);
 const void *reg_kernel_lenient_wide(int K);
+const void *reg_kernel_ext(int K);
 cudaError_t reg_occupancy(const void *func, int warps, size_t smem, int *blocks);
 cudaError_t launch_reg(const RegLaunch &L, const void *func, int grid, size_t smem,
                        cudaStream_t stream);

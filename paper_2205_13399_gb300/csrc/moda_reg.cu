@@ -6,17 +6,20 @@ namespace moda {
 
 const void *reg_kernel_strict(int K, bool narrow) {
   if (!narrow) return reg_kernel_strict_wide(K);
-  return K == 1    ? reinterpret_cast<const void *>(reg_anneal_kernel<1, false, false, false>)
-         : K == 2  ? reinterpret_cast<const void *>(reg_anneal_kernel<2, false, false, false>)
-         : K == 4  ? reinterpret_cast<const void *>(reg_anneal_kernel<4, false, false, true>)
-         : K == 8  ? reinterpret_cast<const void *>(reg_anneal_kernel<8, false, false, true>)
-         : K == 16 ? reinterpret_cast<const void *>(reg_anneal_kernel<16, false, false, true>)
-         : K == 24 ? reinterpret_cast<const void *>(reg_anneal_kernel<24, false, false, true>)
+  return K == 1    ? reinterpret_cast<const void *>(reg_anneal_kernel<1, false, false, false, false>)
+         : K == 2  ? reinterpret_cast<const void *>(reg_anneal_kernel<2, false, false, false, false>)
+         : K == 4  ? reinterpret_cast<const void *>(reg_anneal_kernel<4, false, false, true, false>)
+         : K == 8  ? reinterpret_cast<const void *>(reg_anneal_kernel<8, false, false, true, false>)
+         : K == 16 ? reinterpret_cast<const void *>(reg_anneal_kernel<16, false, false, true, false>)
+         : K == 24 ? reinterpret_cast<const void *>(reg_anneal_kernel<24, false, false, true, false>)
                    : nullptr;
 }
 
-cudaError_t reg_function(int K, bool narrow, bool lenient, int optin, const void **func) {
-  const void *f = lenient ? reg_kernel_lenient(K, narrow) : reg_kernel_strict(K, narrow);
+cudaError_t reg_function(int K, bool narrow, bool lenient, bool ext, int optin,
+                         const void **func) {
+  const void *f = ext       ? reg_kernel_ext(K)
+                  : lenient ? reg_kernel_lenient(K, narrow)
+                            : reg_kernel_strict(K, narrow);
   if (f == nullptr) return cudaErrorInvalidValue;
   // the device's limit, always: launches of one kernel with other sizes may
   // be under way in a graph or on another thread

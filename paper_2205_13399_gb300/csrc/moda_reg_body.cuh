@@ -94,9 +94,15 @@ __device__ __forceinline__ void mma_u8(int32_t (&d)[4], const uint32_t (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-template <int K, bool WIDE, bool LEN, bool INL>
+// EXT carries the options beyond the default algorithm, chosen at run time:
+// normalisation (Sec. 4.2), the offset escape (Alg. 1) and archive snapshots;
+// it takes either acceptance rule and either Delta E range.  Its penalties are
+// floats s_k Delta E_k - E_off, decided by the FP32 test with a margin for
+// their rounding and near it by the double operations as written.
+template <int K, bool WIDE, bool LEN, bool INL, bool EXT>
 __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   static_assert(!INL || K % 4 == 0, "inline draws come four words at a time");
+  static_assert(!EXT || WIDE, "the extensions take either range");
   constexpr bool F64 = reg_f64(K);  // flows as (f1, f2) int32 pairs, else f1 | f2 << 16
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, wid = uni((int)(threadIdx.x >> 5));
@@ -108,7 +114,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   const int row = uni(item.y);
   const int n = uni(R.n), m = uni(R.m), W = uni(R.W), s = uni(R.s), se = uni(R.se);
   const int nc = (m + 127) / 128;
-  if (((uni(R.narrow) != 0) == WIDE) || ((uni(R.accept) != 0) != LEN) || W > G * K) {
+  if ((!EXT && (((uni(R.narrow) != 0) == WIDE) || ((uni(R.accept) != 0) != LEN))) || W > G * K) {
     // the host launches matching variants only
     if (threadIdx.x == 0) atomicExch(R.error, kErrVariant);
     return;
@@ -125,6 +131,20 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   const bool use_mma = uni(R.mma) != 0, fbig = uni(R.fbig) != 0;
   const int dmax = uni(R.dmax);
   auto divn = [&](int p) { return (int)__umulhi((uint32_t)p, magic); };
+  const bool lenient = EXT ? uni(R.accept) != 0 : LEN;
+  const bool norm = EXT && uni(R.normalize) != 0;
+  const bool by_offset = EXT && uni(R.escape) != 0;
+  const double s1 = EXT ? R.s1 : 1.0, s2 = EXT ? R.s2 : 1.0;
+  const float s1f = (float)s1, s2f = (float)s2;
+  const int64_t beta = EXT ? R.beta : 0;
+  const uint32_t snap_every = EXT ? uni((uint32_t)R.snap_every) : 0u;
+  const size_t nsnap = EXT ? (size_t)R.nsnap : 0;
+  // a value no penalty that any draw accepts passes: floor(delta T_max), at
+  // most 2^32 - 1; EXT: the bits of a float above fl(delta T_max)
+  auto top = [&](double delta, int64_t hi) -> uint32_t {
+    if (EXT) return __float_as_uint((float)__dmul_rn(delta, __ldg(&table[0])) * (1.f + 2e-6f));
+    return hi < 0xFFFFFFFFll ? (uint32_t)hi : 0xFFFFFFFFu;
+  };
 
   const RegSmem SL = reg_smem(n, m, se, G, K, WIDE, INL, use_mma);
   constexpr int kFb = F64 ? 8 : 4;       // bytes of a flow pair
@@ -179,9 +199,9 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     RRing e;
     e.delta = R.sch_delta[sn];
     e.cln = accept_scale(e.delta);
-    e.margin = accept_margin(e.delta);
-    const int64_t hi = R.sch_hi[sn];
-    e.hi = hi < 0xFFFFFFFFll ? (uint32_t)hi : 0xFFFFFFFFu;
+    // (EXT: and 1e-6 of the penalty, see ext_penalty)
+    e.margin = accept_margin(e.delta) * (EXT ? 1.6f : 1.f);
+    e.hi = top(e.delta, R.sch_hi[sn]);
     uint32_t c[4] = {0u, q, rep, kTagSelect};
     philox10(c, k0, k1);
     e.sel = c[0];
@@ -259,28 +279,58 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     exact64(k, a1, a2);
     a1 = a1 > 0 ? a1 : 0;
     a2 = a2 > 0 ? a2 : 0;
-    return LEN ? (a1 < a2 ? a1 : a2) : a1 + a2;
+    return lenient ? (a1 < a2 ? a1 : a2) : a1 + a2;
   };
-  // WIDE: the penalty of word k's bit in float, for states whose Delta E pass
+  // WIDE: Delta E of word k's bit in float, for states whose Delta E pass
   // int32: with h > 0 both terms of L + w h are positive, so the sum is within
   // 3 2^-24 of it, else it fits int32 exactly (w < 2^31); the sum of two
   // penalties is within 4 2^-24 (2.8e-6 delta where it is near 11.8 delta,
   // inside the margin of the FP32 test).
-  auto penalty_wide = [&](int k) -> float {
+  auto wide_floats = [&](int k, float &f1, float &f2) {
     const int i = i_of(k), u = u_of(k);
-    if (i >= n) return 3.0e38f;
+    f1 = f2 = 1.0e38f;
+    if (i >= n) return;
     const int x = (int)((xn >> k) & 1u);
     const int h = (int)rcp[i] + (int)rcp[kMaxN + u] - 1 - 2 * x;
     const uint32_t l1 = (x ? 0u - e1[k] : e1[k]) - w1 * (uint32_t)h;
     const uint32_t l2 = (x ? 0u - e2[k] : e2[k]) - w2 * (uint32_t)h;
     const float hf = (float)h;
-    float f1 = h > 0 ? __fmaf_rn(hf, (float)w1, __uint2float_rn(l1))
-                     : __int2float_rn((int32_t)(l1 + w1 * (uint32_t)h));
-    float f2 = h > 0 ? __fmaf_rn(hf, (float)w2, __uint2float_rn(l2))
-                     : __int2float_rn((int32_t)(l2 + w2 * (uint32_t)h));
-    f1 = fmaxf(x ? -f1 : f1, 0.f);
-    f2 = fmaxf(x ? -f2 : f2, 0.f);
-    return LEN ? fminf(f1, f2) : f1 + f2;
+    f1 = h > 0 ? __fmaf_rn(hf, (float)w1, __uint2float_rn(l1))
+               : __int2float_rn((int32_t)(l1 + w1 * (uint32_t)h));
+    f2 = h > 0 ? __fmaf_rn(hf, (float)w2, __uint2float_rn(l2))
+               : __int2float_rn((int32_t)(l2 + w2 * (uint32_t)h));
+    f1 = x ? -f1 : f1;
+    f2 = x ? -f2 : f2;
+  };
+  auto penalty_wide = [&](int k) -> float {
+    float f1, f2;
+    wide_floats(k, f1, f2);
+    f1 = fmaxf(f1, 0.f);
+    f2 = fmaxf(f2, 0.f);
+    return lenient ? fminf(f1, f2) : f1 + f2;
+  };
+  // EXT: the penalty sum_k (min_k) max(0, s_k Delta E_k - E_off) in float.
+  // Near a draw's level each term is at most E_off + 11.8 delta, and its
+  // error at most 6 2^-24 of that (Delta E 3, s_k and the product 2, E_off
+  // 1), so two terms are within 7.2e-7 (E_off + 11.8 delta); the margin adds
+  // 1e-6 (E_off + 12 delta).
+  auto ext_penalty = [&](int k, bool nar, float off) -> float {
+    float f1, f2;
+    if (nar) {
+      f1 = __int2float_rn((int32_t)e1[k]);
+      f2 = __int2float_rn((int32_t)e2[k]);
+    } else if (w1l < (INT64_C(1) << 31) && w2l < (INT64_C(1) << 31)) {
+      wide_floats(k, f1, f2);
+    } else {
+      int64_t x1, x2;
+      exact64(k, x1, x2);
+      f1 = __ll2float_rn(x1);
+      f2 = __ll2float_rn(x2);
+    }
+    f1 = fmaxf(__fmaf_rn(s1f, f1, -off), 0.f);
+    f2 = fmaxf(__fmaf_rn(s2f, f2, -off), 0.f);
+    // (+ 0: never -0, its bits are compared as an integer)
+    return (lenient ? fminf(f1, f2) : f1 + f2) + 0.f;
   };
   const bool wfloat = w1l < (INT64_C(1) << 31) && w2l < (INT64_C(1) << 31);
   auto bits_hm = [&]() {  // WIDE: largest R_i + C_u (one warp)
@@ -547,7 +597,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     while (t <= I_max) {
       __syncthreads();  // A(t): trial t has read its draws
       const int total = __reduce_add_sync(kFull, count_of(t));
-      if (total == 0) {
+      if (total == 0 && !by_offset) {
         __syncthreads();
         __syncthreads();
         const uint32_t mode = uni(sJ[0]);
@@ -578,9 +628,11 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     constexpr bool BAL = K <= 4;
     uint32_t acc[BAL ? K : 1], accb = 0u, amin = 0u;
     int cnt = 0;
+    int64_t Eoff = 0;  // the offset escape's E_off
     auto trial = [&](uint32_t t) {
       const RRing &r = ring[t % kRegRing];
-      const float margin = r.margin;
+      const float off = EXT ? __ll2float_rn(Eoff) : 0.f;
+      const float margin = EXT ? r.margin + 1e-6f * off : r.margin;
       // every |Delta E_k| of the state fits int32 (a bound on the counts that
       // lags by at most three flips, which the limit allows for)
       const bool nar = !WIDE || uni(*reinterpret_cast<volatile int32_t *>(sHm)) <= hm_limit;
@@ -588,7 +640,16 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       float near = 3.0e38f;
       accb = 0u;
       cnt = 0;
-      if (!WIDE || nar) {
+      if (EXT) {
+        float least = 3.0e38f;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          const float v = ext_penalty(k, nar, off);
+          least = fminf(least, v);
+          a[k] = __float_as_uint(v);
+        }
+        amin = nar ? __float_as_uint(least * (1.f - 2e-6f)) : 0u;
+      } else if (!WIDE || nar) {
         amin = 0xFFFFFFFFu;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
@@ -609,7 +670,8 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
           a[k] = __float_as_uint(wfloat ? penalty_wide(k) : penalty_f32(penalty64(k)));
       }
       auto decide = [&](int k, float lv) {
-        const float diff = (!WIDE || nar ? __uint2float_rn(a[k]) : __uint_as_float(a[k])) - lv;
+        const float diff =
+            (!EXT && (!WIDE || nar) ? __uint2float_rn(a[k]) : __uint_as_float(a[k])) - lv;
         near = fminf(near, fabsf(diff));
         if (BAL) {
           const uint32_t b = __ballot_sync(kFull, diff < 0.f);
@@ -625,7 +687,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
 #pragma unroll
         for (int kc = 0; kc < K; kc += 4) {
           bool any = w0 + kc < W;
-          if (any && (!WIDE || nar))
+          if (any && (EXT || !WIDE || nar))
             any = __any_sync(kFull, min(min(a[kc], a[kc + 1]), min(a[kc + 2], a[kc + 3])) <= hi);
           if (any) {
             __syncwarp();  // the last chunk's levels have been read
@@ -657,17 +719,40 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
 #pragma unroll 1
         for (int kk = 0; kk < K; ++kk) {
           uint32_t ak = 0u;
-          int64_t al = 0;
+          int64_t al = 0, x1 = 0, x2 = 0;
 #pragma unroll
           for (int k = 0; k < K; ++k)
             if (k == kk) {
               ak = a[k];
-              if (WIDE && !nar) al = penalty64(k);
+              if (EXT) {
+                if (nar) {
+                  x1 = (int32_t)e1[k];
+                  x2 = (int32_t)e2[k];
+                } else {
+                  exact64(k, x1, x2);
+                }
+              } else if (WIDE && !nar) {
+                al = penalty64(k);
+              }
             }
           const int p = 32 * (w0 + kk) + lane;
           uint32_t d[4] = {(uint32_t)(p >> 2), t, rep, kTagAccept};
           philox10(d, k0, k1);
-          const double ad = WIDE && !nar ? (double)al : (double)ak;
+          double ad = WIDE && !nar ? (double)al : (double)ak;
+          if (EXT && norm) {  // s_1 Delta E_1 (- E_off), ... in IEEE double, as written
+            double y1 = __dmul_rn(s1, (double)x1), y2 = __dmul_rn(s2, (double)x2);
+            if (by_offset) {
+              y1 = __dsub_rn(y1, (double)Eoff);
+              y2 = __dsub_rn(y2, (double)Eoff);
+            }
+            y1 = y1 > 0.0 ? y1 : 0.0;
+            y2 = y2 > 0.0 ? y2 : 0.0;
+            ad = lenient ? (y1 < y2 ? y1 : y2) : __dadd_rn(y1, y2);
+          } else if (EXT) {
+            x1 = x1 > Eoff ? x1 - Eoff : 0;
+            x2 = x2 > Eoff ? x2 - Eoff : 0;
+            ad = (double)(lenient ? (x1 < x2 ? x1 : x2) : x1 + x2);
+          }
           const bool ok = p < m && ad <= __dmul_rn(delta, __ldg(&table[word_of(d, p & 3) >> 16]));
           const uint32_t b = __ballot_sync(kFull, ok);
           cnt += __popc(b);
@@ -698,6 +783,17 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       const uint32_t sums = __reduce_add_sync(kFull, lane < wid ? c | c << 16 : c);
       const int total = (int)(sums & 0xFFFFu), before = (int)(sums >> 16);
       if (lane == 0) sMin[32 * (int)(t & 1u) + wid] = mnw;
+      if (EXT && total == 0 && by_offset) {  // Alg. 1: raise the offset
+        Eoff += beta;
+        if (t == I_max) {
+          __syncthreads();
+          __syncthreads();
+          break;
+        }
+        ++t;
+        trial(t);
+        continue;
+      }
       if (total == 0) {
         __syncthreads();  // the least penalties are complete
         __syncthreads();  // the scan warp has settled the jumps
@@ -753,6 +849,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       }
       if (G > 1) asm volatile("bar.sync 1, %0;" ::"r"(32 * G) : "memory");  // B(t)
       else __syncwarp();
+      if (EXT) Eoff = 0;
       const uint32_t fc = uni(sFlip[t & 3u].code);
       const uint32_t j = fc & 255u, v = (fc >> 8) & 255u;
       const uint32_t sgn = 1u - 2u * (fc >> 16);  // +1: the bit turns on
@@ -808,6 +905,20 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
 
   if (wid == warps - 1) {
     // ================= store warp =================
+    int members = 0;  // |A| as stored
+    // EXT: the states of the snapshots up to iteration `upto`, whose flips are
+    // stored (the scan warp copies the energies)
+    uint32_t snap = snap_every;
+    auto snapshots = [&](uint32_t upto) {
+      for (; EXT && snap_every > 0u && snap <= upto && snap != 0u; snap += snap_every) {
+        const size_t j = snap / snap_every - 1u;
+        if (j >= nsnap) break;
+        uint32_t *to = R.snap_bits + ((size_t)row * nsnap + j) * (size_t)s * W;
+        const int words = members * W;
+#pragma unroll 8
+        for (int q = lane; q < words; q += 32) to[q] = gB[q];
+      }
+    };
     // The state words of the last stored flip in sX; flip tp's follow once
     // its slot is known, an iteration later than the scan warp settles it.
     auto store = [&](uint32_t tp) {
@@ -816,8 +927,10 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       const int fi = (int)(fc & 255u), fu = (int)((fc >> 8) & 255u), ps = fi * n + fu;
       if (lane == 0) sX[ps >> 5] ^= 1u << (ps & 31);
       __syncwarp();
-      if (target >= 0)
+      if (target >= 0) {
         for (int q = lane; q < W; q += 32) gB[(size_t)target * W + q] = sX[q];
+        members = members > target ? members : target + 1;
+      }
       if (WIDE) {
         if (lane == 0) {
           const int sgn = 1 - 2 * (int)(fc >> 16);
@@ -843,14 +956,17 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       __syncthreads();  // A(t)
       const int total = __reduce_add_sync(kFull, count_of(t));
       if (p2) store(t - 2u);
-      if (total > 0) {
+      if (EXT && t > 2u) snapshots(t - 2u);
+      if (total > 0 || by_offset) {
         p2 = p1;
-        p1 = true;
+        p1 = total > 0;
         if (t == I_max) {
           __syncthreads();
           if (p2) store(t - 1u);
+          if (EXT) snapshots(t - 1u);
           __syncthreads();
-          store(t);
+          if (p1) store(t);
+          if (EXT) snapshots(t);
           break;
         }
         refill(t + 2u);
@@ -864,6 +980,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       const uint32_t mode = uni(sJ[0]);
       const int slot = uni((int)sJ[2]);
       t = uni(sJ[1]);
+      if (EXT) snapshots(mode == kRegEnd || mode == kRegStayEnd ? I_max : t - 1u);
       if (mode == kRegEnd || mode == kRegRebuild)  // the member the jumps ended on
         for (int q = lane; q < W; q += 32) sX[q] = gB[(size_t)slot * W + q];  // (written here)
       if (mode == kRegEnd || mode == kRegStayEnd) break;
@@ -893,10 +1010,9 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   }
   const bool exploit = uni(R.archive) != 0;
   int64_t *const trace = R.trace ? R.trace + (size_t)row * (size_t)I_max * 3 : nullptr;
-  const int64_t hiF = R.sch_hi[nsched - 1];
-  const uint32_t hiF32 = hiF < 0xFFFFFFFFll ? (uint32_t)hiF : 0xFFFFFFFFu;
+  const uint32_t hiF32 = top(R.sch_delta[nsched - 1], R.sch_hi[nsched - 1]);
   int acount = 0;
-  uint32_t nflip = 0, njump = 0, nempty = 0, nrebuild = 0;
+  uint32_t nflip = 0, njump = 0, nempty = 0, nrebuild = 0, nraise = 0;
   auto slotE = [&](int y) {
     return y < se ? sAE[y] : make_longlong2(gE[2 * y], gE[2 * y + 1]);
   };
@@ -1001,6 +1117,20 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     return target;
   };
 
+  // EXT: the energies of the snapshots up to iteration `upto`, whose flips are
+  // settled
+  uint32_t snap = snap_every;
+  auto snapshots = [&](uint32_t upto) {
+    for (; EXT && snap_every > 0u && snap <= upto && snap != 0u; snap += snap_every) {
+      const size_t j = snap / snap_every - 1u;
+      if (j >= nsnap) break;
+      const size_t at = (size_t)row * nsnap + j;
+      longlong2 *to = reinterpret_cast<longlong2 *>(R.snap_E) + at * (size_t)s;
+      for (int y = lane; y < acount; y += 32) to[y] = slotE(y);
+      if (lane == 0) R.snap_count[at] = acount;
+    }
+  };
+
   uint32_t t = 1;
   bool pend = false;  // the previous iteration flipped a bit, not settled yet
   int slot_new = -1;  // the slot whose least penalty the last trial gives
@@ -1013,11 +1143,22 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     const int slot_old = slot_new;
     slot_new = pend ? settle(t - 1u) : -1;
     put_min(slot_old, mn);
-    if (flip) {
-      pend = true;
+    if (EXT && t > 1u) snapshots(t - 1u);
+    if (flip || by_offset) {
+      if (EXT && !flip) {
+        ++nraise;
+        if (trace != nullptr && lane == 0) {
+          int64_t *tr = trace + (size_t)(t - 1) * 3;
+          tr[0] = E1;
+          tr[1] = E2;
+          tr[2] = INT64_MIN;
+        }
+      }
+      pend = flip;
       if (t == I_max) {
         __syncthreads();
-        settle(t);
+        if (flip) settle(t);
+        if (EXT) snapshots(t);
         __syncthreads();
         break;
       }
@@ -1038,6 +1179,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       }
       ++nempty;
       const bool end = t == I_max;
+      if (EXT) snapshots(t);
       if (!end) ++t;
       if (lane == 0) {
         sJ[0] = end ? kRegStayEnd : kRegStay;  // sX still holds the state
@@ -1084,8 +1226,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
         if (it + 1u <= ring_to) {
           hi = ring[(it + 1u) % kRegRing].hi;
         } else if (it + 1u < nsched) {
-          const int64_t h = R.sch_hi[it];
-          hi = h < 0xFFFFFFFFll ? (uint32_t)h : 0xFFFFFFFFu;
+          hi = top(R.sch_delta[it], R.sch_hi[it]);
         }
       }
       const unsigned stop = __ballot_sync(kFull, last || mn <= hi);
@@ -1106,6 +1247,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       }
       t += 32u;
     }
+    if (EXT) snapshots(end ? I_max : t - 1u);
     if (lane == 0) {
       sJ[0] = end ? kRegEnd : kRegRebuild;
       sJ[1] = t;
@@ -1137,7 +1279,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     st[0] = nflip;
     st[1] = njump;
     st[2] = nempty;
-    st[3] = 0;
+    st[3] = nraise;
     st[4] = 0;
     st[5] = (int64_t)njump - (int64_t)nrebuild;
     st[6] = 0;

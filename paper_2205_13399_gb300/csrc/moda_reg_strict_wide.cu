@@ -5,10 +5,10 @@
 namespace moda {
 
 const void *reg_kernel_strict_wide(int K) {
-  return K == 4    ? reinterpret_cast<const void *>(reg_anneal_kernel<4, true, false, true>)
-         : K == 8  ? reinterpret_cast<const void *>(reg_anneal_kernel<8, true, false, true>)
-         : K == 16 ? reinterpret_cast<const void *>(reg_anneal_kernel<16, true, false, true>)
-         : K == 24 ? reinterpret_cast<const void *>(reg_anneal_kernel<24, true, false, true>)
+  return K == 4    ? reinterpret_cast<const void *>(reg_anneal_kernel<4, true, false, true, false>)
+         : K == 8  ? reinterpret_cast<const void *>(reg_anneal_kernel<8, true, false, true, false>)
+         : K == 16 ? reinterpret_cast<const void *>(reg_anneal_kernel<16, true, false, true, false>)
+         : K == 24 ? reinterpret_cast<const void *>(reg_anneal_kernel<24, true, false, true, false>)
                    : nullptr;
 }
 

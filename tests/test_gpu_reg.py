@@ -101,3 +101,67 @@ def test_accept_every_draw():
             assert np.array_equal(acc, a.astype(np.float64) <= prod), (k, off)
             if abs(off) < 2e-5 and delta > 1e6:
                 assert (path == -1).all()
+
+
+# the extensions: 12 one word a worker, 30 two, 40 four, 56 eight
+@pytest.mark.parametrize("n", [3, 12, 30, 40, 56])
+@pytest.mark.parametrize("esc", ["archive", "offset"])
+@pytest.mark.parametrize("norm", [False, True])
+@pytest.mark.parametrize("acc,arc", [("strict", "explore"), ("lenient", "exploit")])
+def test_extensions_traced(n, esc, norm, acc, arc):
+    if esc == "archive" and not norm:
+        pytest.skip("the default algorithm")
+    inst = inputs.uniform_instance(n, index=60 + n, workload="P8")
+    kw = dict(replicas=2, I_max=900, seed=n, accept=acc, archive=arc, escape=esc, beta=30_000)
+    # Sec. 4.2's units are larger: a schedule that reaches the frozen phase in both
+    kw.update(dict(delta0=3e8, deltaf=1e6, xi=0.02) if norm else FAST)
+    _, _, res, tr = gpu_run(inst, trace=True, normalize=norm, **kw)
+    _, orc = oracle_run(inst, trace=True, normalize=norm, **kw)
+    compare(res, range(2), orc, n * n, gpu_trace=tr)
+    if esc == "offset" and n <= 30:  # (larger ones are still descending after 900 flips)
+        assert res.stats[:, 3].sum() > 0
+
+
+@pytest.mark.parametrize("esc", ["archive", "offset"])
+@pytest.mark.parametrize("norm", [False, True])
+def test_extensions_beyond_int32(esc, norm):
+    if esc == "archive" and not norm:
+        pytest.skip("the default algorithm")
+    n = 41
+    rng = np.random.default_rng(n)
+    F1, F2 = (rng.integers(300, 900, (n, n)) for _ in range(2))
+    inst = _Inst(F1, F2, rng.integers(50, 120, (n, n)))
+    kw = dict(replicas=2, I_max=2500, seed=3, escape=esc, beta=4_000_000, delta0=1e10, deltaf=1e6,
+              xi=5e-3)
+    _, _, res, tr = gpu_run(inst, trace=True, normalize=norm, **kw)
+    _, orc = oracle_run(inst, trace=True, normalize=norm, **kw)
+    compare(res, range(2), orc, n * n, gpu_trace=tr)
+
+
+@pytest.mark.parametrize("K", [1, 7, 250, 600])
+@pytest.mark.parametrize("esc", ["archive", "offset"])
+def test_snapshots(K, esc):
+    """Snapshots at every spacing: after flips, inside runs of jumps, at the
+    last iteration."""
+    from paper_2205_13399_gb300 import moda
+    n, R, I_max = 9, 2, 600
+    inst = inputs.uniform_instance(n, index=5, workload="P8")
+    kw = dict(replicas=R, I_max=I_max, seed=2, escape=esc, beta=2000, **FAST)
+    g = moda.Instance(inst.F1, inst.F2, inst.D)
+    run = moda.anneal(g, snapshot_every=K, **kw).wait()
+    _, orc = oracle_run(inst, snapshot_every=K, **kw)
+    snap = orc["snapshots"]
+    for r in range(R):
+        for j in range(0, I_max // K, max(1, I_max // K // 40)):
+            c = int(snap["count"][r, j])
+            E = snap["E"][r, j, :c]
+            pts = [(int(a), int(b)) for a, b in E]
+            want = sorted(pts[i] for i in oracle.nondominated(pts))
+            got = run.read_archive(replica=r, snapshot=j)
+            assert [(p["E1"], p["E2"]) for p in got] == want, (r, j)
+            for p in got:
+                slot = p["slot"]
+                assert pts[slot] == (p["E1"], p["E2"])
+                if p["perm"] is not None:
+                    assert p["perm"] == oracle.decode_permutation(snap["bits"][r, j, slot])
+    compare(run.read(), range(R), orc, n * n)
