@@ -347,60 +347,13 @@ int warp_slots(moda_instance inst, const moda_params &p) {
 // Archive energies kept in shared memory per warp, at most.
 constexpr int kWarpSmemEnergies = 512;
 
-// Archive slots the register annealer keeps on chip (energies and least
-// penalties), at most: the archives of the workloads reach 528 members.
-constexpr int kRegSlots = 768;
-
-// How a run fits the register annealer at K words per worker: its archive
-// slots on chip (0: it cannot run so) and whether rebuilds use matrix
-// products.  Its packed rows hold 16-bit flows, and everything but the slots
-// must fit in shared memory.
-struct RegFit {
-  int se = 0;
-  bool mma = false;
-};
-RegFit reg_fit(moda_instance inst, int s, int K, bool wide, int optin) {
-  RegFit f;
-  const int workers = (inst->W + K - 1) / K;
-  if (inst->fmax > 65535 || inst->dmax > 65535 || workers > moda::kRegMaxWorkers) return f;
-  for (const bool mma : {2 * inst->dmax <= 65535, false})
-    for (int se = std::min(s, kRegSlots); se >= 1; se = se > 64 ? se / 2 : se / 8)
-      if ((int64_t)moda::reg_smem(inst->n, inst->m, se, workers, K, wide, K >= 4, mma).total <=
-          optin) {
-        f.se = se;
-        f.mma = mma;
-        return f;
-      }
-  return f;
-}
-
-// The words per worker that suit a run best where its launch has the device
-// to itself as far as it can (crowded: no): few words shorten an iteration,
-// and up to n = 35 draw warps take Philox off the workers (draws: the kernel
-// has such variants).
-int reg_words(int W, bool draws, bool crowded) {
-  if (!crowded) {
-    if (draws && W <= 20) return 1;
-    if (draws && W <= 40) return 2;
-    if (W <= 88) return 4;
-    if (W <= 176) return 8;
-  }
-  return W <= 32 ? 4 : W <= 96 ? 8 : W <= 16 * moda::kRegMaxWorkers ? 16 : 24;
-}
-
-// reg_fit at either choice of words per worker (the launch is planned
-// later): the smaller of the slot counts.
-RegFit reg_plan(moda_instance inst, const moda_params *p, bool narrow) {
+// How a request fits the register annealer (se = 0: it does not).
+moda::RegFit reg_plan(moda_instance inst, const moda_params *p, bool narrow) {
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, inst->device);
-  const bool ext = !warp_options(p);
-  const int s = p->archive_size > 0 ? p->archive_size : inst->m;
-  const bool draws = narrow || ext, wide = !narrow || ext;
-  RegFit f = reg_fit(inst, s, reg_words(inst->W, draws, false), wide, optin);
-  const RegFit g = reg_fit(inst, s, reg_words(inst->W, draws, true), wide, optin);
-  f.se = std::min(f.se, g.se);
-  f.mma = f.mma && g.mma;
-  return f;
+  return moda::reg_fit(inst->n, inst->fmax, inst->dmax,
+                       p->archive_size > 0 ? p->archive_size : inst->m, narrow, !warp_options(p),
+                       optin);
 }
 
 // Whether a warp-engine request prescribes the team annealer's layout (team
@@ -612,7 +565,7 @@ moda_status prepare_warp_run(moda_instance inst, const moda_params *p, cudaStrea
   r->stream = stream;
   r->warp = true;
   const bool narrow = moda::narrow_ok(inst->n, inst->b1, inst->b2, inst->w1, inst->w2);
-  RegFit fit;
+  moda::RegFit fit;
   if (!prescribes_team(p)) fit = reg_plan(inst, p, narrow);
   r->reg = fit.se > 0;
   const size_t R = r->R, s = r->s, W = inst->W;
@@ -672,15 +625,7 @@ moda_status prepare_warp_run(moda_instance inst, const moda_params *p, cudaStrea
   w.fbig = inst->fmax > 255 ? 1 : 0;
   w.dmax = (int32_t)std::min<int64_t>(inst->dmax, 65535);
   w.arch_min = r->arch_min;
-  {
-    // |Delta E_k| <= B_k + w_k (R_i + C_u + 1); the device's largest
-    // R_i + C_u lags by at most three flips (6)
-    int64_t lim = 1 << 20;
-    const int64_t b[2] = {inst->b1, inst->b2}, ww[2] = {inst->w1, inst->w2};
-    for (int k = 0; k < 2; ++k)
-      if (ww[k] > 0) lim = std::min(lim, (INT64_C(2147483646) - b[k]) / ww[k] - 8);
-    w.hm_limit = (int32_t)std::max<int64_t>(lim, -1);
-  }
+  w.hm_limit = moda::reg_hm_limit(inst->b1, inst->b2, inst->w1, inst->w2);
   w.normalize = p->normalize;
   w.escape = p->escape;
   w.beta = p->beta;
@@ -1025,10 +970,8 @@ moda_status plan_reg_group(std::vector<moda_run> &runs, std::vector<Prepared> &p
   std::vector<moda::WarpRun> descs;
   std::vector<std::pair<int, int>> order;  // (-m, k): largest first
   std::vector<int2> items;
-  int W = 1;
   for (size_t k = 0; k < G.idx.size(); ++k) {
     const moda_run r = runs[G.idx[k]];
-    W = std::max(W, r->inst->W);
     descs.push_back(pls[G.idx[k]].wrun);
     order.emplace_back(-r->inst->m, (int)k);
   }
@@ -1039,40 +982,10 @@ moda_status plan_reg_group(std::vector<moda_run> &runs, std::vector<Prepared> &p
   MODA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, r0->inst->device));
   MODA_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin,
                                    r0->inst->device));
-  // The fewest words per worker whose blocks are all resident at once, else
-  // the choice for a crowded device.
-  int K = 0, workers = 0, draws = 0;
-  size_t smem = 0;
-  const bool ext = !warp_options(&r0->prm), wide = !narrow || ext, draw_warps = narrow || ext;
-  const int crowded = reg_words(W, draw_warps, true);
-  for (int c = reg_words(W, draw_warps, false); K == 0; c = c < 8 ? 2 * c : c + 8) {
-    if (c < 4 && crowded < c) continue;
-    const int g = (W + c - 1) / c, d = c < 4 ? (W + 3) / 4 : 0;
-    const bool inl = c >= 4;
-    size_t need = 0;
-    for (const moda::WarpRun &w : descs)
-      need = std::max<size_t>(
-          need, moda::reg_smem(w.n, w.m, w.se, g, c, wide, inl, w.mma != 0).total);
-    const void *func = nullptr;
-    int blocks = 0;
-    if (g <= moda::kRegMaxWorkers && (draw_warps || inl) && need <= (size_t)optin) {
-      cudaError_t e = moda::reg_function(c, narrow, r0->prm.accept != 0, ext, optin, &func);
-      if (e == cudaSuccess) e = moda::reg_occupancy(func, g + d + 2, need, &blocks);
-      if (e != cudaSuccess) {
-        cudaGetLastError();
-        blocks = 0;
-      }
-    }
-    if (blocks >= 1 && ((int64_t)blocks * sms >= (int64_t)items.size() || c >= crowded)) {
-      K = c;
-      workers = g;
-      draws = d;
-      smem = need;
-      G.func = func;
-    } else if (c >= 24) {
-      return fail(MODA_EUNSUPPORTED, "register annealer: the run does not fit a block");
-    }
-  }
+  moda::RegChoice c;
+  MODA_CUDA(moda::reg_choose(descs.data(), (int)descs.size(), (int64_t)items.size(),
+                             !warp_options(&r0->prm), sms, optin, &c));
+  if (c.K == 0) return fail(MODA_EUNSUPPORTED, "register annealer: the run does not fit a block");
   auto scratch = std::make_shared<WarpScratch>();
   scratch->device = r0->inst->device;
   // on failure after this point, work already enqueued may still use the
@@ -1095,17 +1008,18 @@ moda_status plan_reg_group(std::vector<moda_run> &runs, std::vector<Prepared> &p
     moda_run r = runs[k];
     MODA_CUDA(cudaMemsetAsync(r->error, 0, sizeof(int32_t), stream));
     r->wscratch = scratch;
-    r->threads = workers;
+    r->threads = c.workers;
     r->bpt = (int)items.size();
   }
   G.reg = true;
   G.narrow = narrow;
   G.RL.runs = reinterpret_cast<const moda::WarpRun *>(base);
   G.RL.items = reinterpret_cast<const int2 *>(base + d_bytes);
-  G.RL.workers = workers;
-  G.RL.draws = draws;
+  G.RL.workers = c.workers;
+  G.RL.draws = c.draws;
+  G.func = c.func;
   G.grid = (int)items.size();
-  G.smem = smem;
+  G.smem = c.smem;
   G.scratch = scratch;
   guard.armed = false;
   return MODA_OK;
@@ -1736,7 +1650,7 @@ moda_status moda_anneal_batch(const moda_instance *insts, const moda_params *par
     if (!runs[i]->warp) continue;
     const int nc = (runs[i]->inst->m + 127) / 128;
     if (runs[i]->reg) {
-      const int K = reg_words(runs[i]->inst->W, true, true);
+      const int K = moda::reg_words(runs[i]->inst->W, true, true);
       const bool ext = !warp_options(&runs[i]->prm);
       classes[std::make_tuple(-K * 100 - (runs[i]->inst->W + K - 1) / K, 1,
                               ext ? 2 : pls[i].narrow ? 1 : 0, ext ? 0 : runs[i]->prm.accept)]

@@ -438,10 +438,20 @@ constexpr int kRegMaxWorkers = 26;
 
 // Flow pairs as two int32 (fewer instructions) where they are small.
 __host__ __device__ constexpr bool reg_f64(int K) { return K <= 8; }
+// Pairs of a flow row: n, at least one zero, and a stride that is 2 words
+// modulo 8, so that the lanes of a matrix fragment (8 facilities by 4 rows,
+// four rows apart) hit different banks.
+__host__ __device__ inline int reg_fcols(int n, bool f64) {
+  const int mod = f64 ? 4 : 8, want = f64 ? 1 : 2;
+  return n + 1 + ((want - (n + 1)) % mod + mod) % mod;
+}
 // Registers per thread: what K words of Delta E need without spilling in the
-// flip's round, and as many resident blocks as that leaves.
+// flip's round, and as many resident blocks as that leaves (K = 4 serves
+// crowded launches: 64 registers keep two blocks of 15 warps on an SM, 131 ms
+// for 1,500 replicas of n = 40 against 186 ms with 72; K = 1 and 2 run one
+// block an SM, where 64 spilled: 5.0 ms against 4.2 on n = 8).
 __host__ __device__ constexpr int reg_regs(int K) {
-  return K <= 4 ? 64 : K == 8 ? 80 : K == 16 ? 72 : 96;
+  return K <= 2 ? 72 : K == 4 ? 64 : K == 8 ? 80 : K == 16 ? 72 : 96;
 }
 
 // Rebuild by matrix products (flag mma of a run): M^T as bytes, one row per
@@ -458,7 +468,7 @@ __host__ __device__ inline RegSmem reg_smem(int n, int m, int se, int workers, i
   const int nc = (m + 127) / 128;
   RegSmem L;
   size_t o = 0;
-  L.fs = 0;              o = align_up((size_t)(reg_f64(K) ? 8 : 4) * n * (n + 1), 16);
+  L.fs = 0;              o = align_up((size_t)(reg_f64(K) ? 8 : 4) * n * reg_fcols(n, reg_f64(K)), 16);
   L.d = (uint32_t)o;     o = align_up(o + 4 * (size_t)m, 16);
   L.ring = (uint32_t)o;  o = align_up(o + 32 * (size_t)kRegRing, 16);
   L.cnt = (uint32_t)o;   o = align_up(o + 4 * 2 * 32, 16);
@@ -486,10 +496,47 @@ __host__ __device__ inline RegSmem reg_smem(int n, int m, int se, int workers, i
 
 struct RegLaunch {
   const WarpRun *runs;
-  const int2 *items;  // (run, replica row), one block each, largest runs first
+  const int2 *items;  // (run, replica row), one block each, largest runs first;
+                      // nullptr: block b runs replica b of the only run
   int32_t workers;    // G
   int32_t draws;      // D (0 with inline draws)
 };
+
+// Archive slots kept on chip (energies and least penalties), at most: the
+// archives of the workloads reach 528 members.
+constexpr int kRegSlots = 768;
+
+// The words per worker that suit a run of W state words best where its launch
+// has the device to itself as far as it can (crowded: no): few words shorten
+// an iteration, and up to n = 35 draw warps take Philox off the workers
+// (draws: the kernel has such variants).
+int reg_words(int W, bool draws, bool crowded);
+
+// How a run fits the register annealer, at either choice of words per worker
+// (the launch is planned later): its archive slots on chip (0: it cannot run
+// there) and whether rebuilds use matrix products.  Flows are packed as 16
+// bits, and everything but the slots must fit in shared memory.
+struct RegFit {
+  int se = 0;
+  bool mma = false;
+};
+RegFit reg_fit(int n, int64_t fmax, int64_t dmax, int s, bool narrow, bool ext, int optin);
+
+// The largest max_i R_i + max_u C_u at which every Delta E_k surely fits
+// int32 (WarpRun::hm_limit): |Delta E_k| <= B_k + w_k (R_i + C_u + 1), and the
+// device's value lags by at most three flips (6).
+int32_t reg_hm_limit(int64_t b1, int64_t b2, int64_t w1, int64_t w2);
+
+// The launch shape for `items` replicas of the `count` runs: the fewest words
+// per worker whose blocks are all resident at once, else the choice for a
+// crowded device.  K = 0: no shape fits.
+struct RegChoice {
+  int K = 0, workers = 0, draws = 0;
+  size_t smem = 0;
+  const void *func = nullptr;
+};
+cudaError_t reg_choose(const WarpRun *runs, int count, int64_t items, bool ext, int sms, int optin,
+                       RegChoice *out);
 
 // The kernel with K words per worker (1, 2 with draw warps and int32 Delta E
 // only; 4, 8, 16, 24 with inline draws), with `optin` bytes of dynamic shared

@@ -48,6 +48,7 @@ static __device__ __align__(256) int64_t g_sched_hi[kSchedMax];
 static __device__ __align__(256) int32_t g_fs1[kNN];
 static __device__ __align__(256) int32_t g_fs2[kNN];
 static __device__ __align__(256) int32_t g_d[kNN];
+static __device__ __align__(256) unsigned char g_run[sizeof(moda::WarpRun)];
 
 struct DeviceSymbols {
   bool ready = false;
@@ -56,6 +57,7 @@ struct DeviceSymbols {
   float *tablef = nullptr;
   int64_t *lo = nullptr, *hi = nullptr;
   int32_t *fs1 = nullptr, *fs2 = nullptr, *d = nullptr;
+  moda::WarpRun *run = nullptr;
   double tmin = 0, tmax = 0;
 };
 
@@ -68,6 +70,7 @@ float h_tablef[moda::kTableSize];
 double h_delta[kSchedMax];
 int64_t h_lo[kSchedMax], h_hi[kSchedMax];
 int32_t h_fs1[kNN], h_fs2[kNN], h_d[kNN];
+moda::WarpRun h_run;
 
 moda_status nofail(moda_status st, const std::string &msg) {
   moda::set_last_error(msg);
@@ -93,6 +96,7 @@ moda_status setup(int dev, DeviceSymbols **out) {
     if (e == cudaSuccess) e = symbol(&S.fs1, g_fs1);
     if (e == cudaSuccess) e = symbol(&S.fs2, g_fs2);
     if (e == cudaSuccess) e = symbol(&S.d, g_d);
+    if (e == cudaSuccess) e = symbol(&S.run, g_run);
     if (e != cudaSuccess)
       return nofail(MODA_ECUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
     for (int idx = 0; idx < moda::kTableSize; ++idx)
@@ -283,6 +287,79 @@ extern "C" moda_status moda_anneal_noalloc(int32_t n, const int16_t *F1,
     return nofail(MODA_ECUDA, std::string("upload: ") + cudaGetErrorString(e));
   // The host staging arrays are pageable: each copy has read them before
   // cudaMemcpyAsync returns, so the next call may reuse them.
+
+  // The register annealer (as moda_anneal with the engine left open) unless
+  // the request prescribes the block engine or its fast-forward, or the
+  // least penalties of archive slots off chip do not fit the scratch array.
+  if (p->engine != 1 && p->block_threads == 0 && !p->fast_forward) {
+    const bool ext = p->escape != MODA_ESC_ARCHIVE || p->normalize != 0;
+    const moda::RegFit fit =
+        moda::reg_fit(n, std::max(e1max, e2max), edmax, s, narrow, ext, dev_smem);
+    const bool spill = s > fit.se;  // least penalties off chip
+    if (fit.se > 0 &&
+        (!spill || (size_t)p->replicas * (size_t)s * sizeof(uint32_t) <= kScratchBytes)) {
+      moda::WarpRun &w = h_run;
+      w = moda::WarpRun{};
+      w.n = n;
+      w.m = m;
+      w.W = W;
+      w.s = s;
+      w.se = fit.se;
+      w.mma = fit.mma ? 1 : 0;
+      w.fbig = std::max(e1max, e2max) > 255 ? 1 : 0;
+      w.dmax = (int32_t)edmax;
+      w.arch_min = spill ? reinterpret_cast<uint32_t *>(S->scratch) : nullptr;
+      w.hm_limit = moda::reg_hm_limit(f1max * dmax, f2max * dmax, w1, w2);
+      w.narrow = narrow ? 1 : 0;
+      w.accept = p->accept;
+      w.archive = p->archive;
+      w.normalize = p->normalize;
+      w.escape = p->escape;
+      w.s1 = p->normalize ? moda::norm_scale(e1max * edmax) : 1.0;
+      w.s2 = p->normalize ? moda::norm_scale(e2max * edmax) : 1.0;
+      w.beta = p->beta;
+      w.nsched = nsched;
+      w.replicas = p->replicas;
+      w.replica_base = (uint32_t)p->replica_base;
+      w.seed_lo = (uint32_t)(p->seed & 0xFFFFFFFFull);
+      w.seed_hi = (uint32_t)(p->seed >> 32);
+      w.magic = (uint32_t)(0xFFFFFFFFu / (uint32_t)n) + 1u;
+      w.I_max = p->I_max;
+      w.w1 = w1;
+      w.w2 = w2;
+      w.sch_delta = S->delta;
+      w.sch_lo = S->lo;
+      w.sch_hi = S->hi;
+      w.table = S->table;
+      w.tablef = S->tablef;
+      w.Fs1 = S->fs1;
+      w.Fs2 = S->fs2;
+      w.D = S->d;
+      w.arch_E = out->arch_E;
+      w.arch_bits = out->arch_bits;
+      w.arch_count = out->arch_count;
+      w.x_final = out->x_final;
+      w.E_final = out->E_final;
+      w.stats = out->stats;
+      w.error = out->error;
+      int sms = 1;
+      e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+      moda::RegChoice c;
+      if (e == cudaSuccess) e = moda::reg_choose(&w, 1, p->replicas, ext, sms, dev_smem, &c);
+      if (e == cudaSuccess && c.K > 0) {
+        e = cudaMemcpyAsync(S->run, &w, sizeof(w), cudaMemcpyHostToDevice, stream);
+        moda::RegLaunch L{};
+        L.runs = S->run;
+        L.items = nullptr;
+        L.workers = c.workers;
+        L.draws = c.draws;
+        if (e == cudaSuccess) e = moda::launch_reg(L, c.func, p->replicas, c.smem, stream);
+        if (e == cudaSuccess) return MODA_OK;
+      }
+      if (e != cudaSuccess)
+        return nofail(MODA_ECUDA, std::string("launch: ") + cudaGetErrorString(e));
+    }
+  }
 
   moda::AnnealArgs a{};
   a.n = n;

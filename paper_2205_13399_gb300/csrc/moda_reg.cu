@@ -1,5 +1,7 @@
 // Register annealer, strict acceptance, Delta E within int32 (see
-// moda_reg_body.cuh), and the launch of every variant.
+// moda_reg_body.cuh), and the choice and launch of every variant.
+#include <algorithm>
+
 #include "moda_reg_body.cuh"
 
 namespace moda {
@@ -26,6 +28,78 @@ cudaError_t reg_function(int K, bool narrow, bool lenient, bool ext, int optin,
   cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
   if (e == cudaSuccess) *func = f;
   return e;
+}
+
+// Uncrowded, measured on n = 8: 4.2 ms with one word, 4.8 with two; n = 25
+// (128 replicas): 14.4, 13.7 and 14.6 ms with one, two and four; n = 33: four
+// and two alike, eight a fifth slower; n = 75: 67 ms with eight, 113 with 16.
+// Crowded: n = 20 97 ms with four, 138 with eight; n = 40 131 and 165; n = 60
+// 235 with eight, 293 with 16 (72 registers spill there).
+int reg_words(int W, bool draws, bool crowded) {
+  if (!crowded) {
+    if (draws && W <= 8) return 1;
+    if (draws && W <= 40) return 2;
+    if (W <= 88) return 4;
+    if (W <= 176) return 8;
+  }
+  return W <= 56 ? 4 : W <= 176 ? 8 : W <= 16 * kRegMaxWorkers ? 16 : 24;
+}
+
+RegFit reg_fit(int n, int64_t fmax, int64_t dmax, int s, bool narrow, bool ext, int optin) {
+  const int m = n * n, W = (m + 31) / 32;
+  const bool wide = !narrow || ext, draws = narrow || ext;
+  RegFit f{kRegSlots, true};
+  if (fmax > 65535 || dmax > 65535) return RegFit{};
+  for (const bool crowded : {false, true}) {
+    const int K = reg_words(W, draws, crowded), workers = (W + K - 1) / K;
+    if (workers > kRegMaxWorkers) return RegFit{};
+    RegFit g;
+    for (const bool mma : {2 * dmax <= 65535, false})
+      for (int se = std::min(s, kRegSlots); se >= 1 && g.se == 0; se = se > 64 ? se / 2 : se / 8)
+        if ((int64_t)reg_smem(n, m, se, workers, K, wide, K >= 4, mma).total <= optin)
+          g = RegFit{se, mma};
+    f.se = std::min(f.se, g.se);
+    f.mma = f.mma && g.mma;
+  }
+  return f;
+}
+
+int32_t reg_hm_limit(int64_t b1, int64_t b2, int64_t w1, int64_t w2) {
+  int64_t lim = 1 << 20;
+  const int64_t b[2] = {b1, b2}, w[2] = {w1, w2};
+  for (int k = 0; k < 2; ++k)
+    if (w[k] > 0) lim = std::min<int64_t>(lim, (INT64_C(2147483646) - b[k]) / w[k] - 8);
+  return (int32_t)std::max<int64_t>(lim, -1);
+}
+
+cudaError_t reg_choose(const WarpRun *runs, int count, int64_t items, bool ext, int sms, int optin,
+                       RegChoice *out) {
+  *out = RegChoice{};
+  int W = 1;
+  for (int k = 0; k < count; ++k) W = std::max(W, runs[k].W);
+  const bool narrow = runs[0].narrow != 0, wide = !narrow || ext, draws = narrow || ext;
+  const int crowded = reg_words(W, draws, true);
+  for (int K = reg_words(W, draws, false); K <= 24; K = K < 8 ? 2 * K : K + 8) {
+    const int g = (W + K - 1) / K, d = K < 4 ? std::min((W + 3) / 4, 6) : 0;
+    const bool inl = K >= 4;
+    size_t need = 0;
+    for (int k = 0; k < count; ++k)
+      need = std::max<size_t>(need, reg_smem(runs[k].n, runs[k].m, runs[k].se, g, K, wide, inl,
+                                             runs[k].mma != 0)
+                                        .total);
+    if (g > kRegMaxWorkers || need > (size_t)optin) continue;
+    const void *func = nullptr;
+    cudaError_t e = reg_function(K, narrow, runs[0].accept != 0, ext, optin, &func);
+    if (e != cudaSuccess) return e;
+    int blocks = 0;
+    e = reg_occupancy(func, g + d + 2, need, &blocks);
+    if (e != cudaSuccess) return e;
+    if (blocks >= 1 && ((int64_t)blocks * sms >= items || K >= crowded)) {
+      *out = RegChoice{K, g, d, need, func};
+      return cudaSuccess;
+    }
+  }
+  return cudaSuccess;
 }
 
 cudaError_t reg_occupancy(const void *func, int warps, size_t smem, int *blocks) {

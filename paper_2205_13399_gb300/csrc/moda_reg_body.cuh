@@ -109,7 +109,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   const int G = L.workers, D = INL ? 0 : L.draws;
   const int warps = G + D + 2, threads = 32 * warps;
   const bool worker = wid < G;
-  const int2 item = L.items[blockIdx.x];
+  const int2 item = L.items != nullptr ? L.items[blockIdx.x] : make_int2(0, (int)blockIdx.x);
   const WarpRun &R = L.runs[item.x];
   const int row = uni(item.y);
   const int n = uni(R.n), m = uni(R.m), W = uni(R.W), s = uni(R.s), se = uni(R.se);
@@ -148,7 +148,8 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
 
   const RegSmem SL = reg_smem(n, m, se, G, K, WIDE, INL, use_mma);
   constexpr int kFb = F64 ? 8 : 4;       // bytes of a flow pair
-  const int frow = (n + 1) * kFb;        // bytes of a flow row: n pairs and a zero
+  const int fcols = reg_fcols(n, F64);
+  const int frow = fcols * kFb;          // bytes of a flow row: n pairs and zeros
   unsigned char *const sFs = smem + SL.fs;
   unsigned char *const sD = smem + SL.d;
   RRing *const ring = reinterpret_cast<RRing *>(smem + SL.ring);
@@ -169,8 +170,8 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   uint32_t *const sAM = reinterpret_cast<uint32_t *>(smem + SL.aM);    // least penalties
 
   // ---- matrices, ring, initial state (R10) into shared memory
-  for (int e = threadIdx.x; e < n * (n + 1); e += threads) {
-    const int j = e / (n + 1), i = e - j * (n + 1);
+  for (int e = threadIdx.x; e < n * fcols; e += threads) {
+    const int j = e / fcols, i = e - j * fcols;
     const int32_t f1 = i < n ? R.Fs1[j * n + i] : 0, f2 = i < n ? R.Fs2[j * n + i] : 0;
     if (F64) reinterpret_cast<int2 *>(sFs)[e] = make_int2(f1, f2);
     else reinterpret_cast<uint32_t *>(sFs)[e] = (uint32_t)f1 | ((uint32_t)f2 << 16);
@@ -404,18 +405,22 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       }
       __syncthreads();
       // ---- strips of 16 rows: every warp takes tiles of 8 columns; A is
-      // Fs (symmetric: flow row j, split into bytes by permutes), the
-      // products of byte planes add up shifted by their weights
+      // Fs (symmetric: flow row j, split into bytes by permutes; the stride
+      // of a flow row keeps a fragment's loads free of bank conflicts, which
+      // were 4-way without it), the products of byte planes add up shifted
+      // by their weights
       int2 *const sL = reinterpret_cast<int2 *>(smem + SL.scr);
       const int gi = lane >> 2, ti = lane & 3;
       for (int ib = 0; ib < n; ib += 16) {
         for (int ut = 8 * wid; ut < n; ut += 8 * warps) {
           uint32_t l1[4] = {0u, 0u, 0u, 0u}, l2[4] = {0u, 0u, 0u, 0u};
-          for (int mp = 0; mp <= (mbig ? 1 : 0); ++mp) {
+#pragma unroll 1
+          for (int mp = 0; mp <= (mbig ? 1 : 0); ++mp) {  // the byte of M
             const unsigned char *bm = (mp ? mhi : mlo) + (ut + gi) * ms + 4 * ti;
             int32_t c[4][4];
 #pragma unroll
             for (int f = 0; f < 4; ++f) c[f][0] = c[f][1] = c[f][2] = c[f][3] = 0;
+#pragma unroll 1
             for (int kb = 0; kb < n; kb += 32) {
               uint32_t a[4][4];  // [plane][fragment register]
 #pragma unroll
@@ -910,13 +915,16 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     // stored (the scan warp copies the energies)
     uint32_t snap = snap_every;
     auto snapshots = [&](uint32_t upto) {
-      for (; EXT && snap_every > 0u && snap <= upto && snap != 0u; snap += snap_every) {
-        const size_t j = snap / snap_every - 1u;
-        if (j >= nsnap) break;
-        uint32_t *to = R.snap_bits + ((size_t)row * nsnap + j) * (size_t)s * W;
-        const int words = members * W;
+      if constexpr (EXT) {
+        if (snap_every == 0u) return;
+        for (; snap <= upto && snap != 0u; snap += snap_every) {
+          const size_t j = snap / snap_every - 1u;
+          if (j >= nsnap) break;
+          uint32_t *to = R.snap_bits + ((size_t)row * nsnap + j) * (size_t)s * W;
+          const int words = members * W;
 #pragma unroll 8
-        for (int q = lane; q < words; q += 32) to[q] = gB[q];
+          for (int q = lane; q < words; q += 32) to[q] = gB[q];
+        }
       }
     };
     // The state words of the last stored flip in sX; flip tp's follow once
@@ -1121,13 +1129,16 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   // settled
   uint32_t snap = snap_every;
   auto snapshots = [&](uint32_t upto) {
-    for (; EXT && snap_every > 0u && snap <= upto && snap != 0u; snap += snap_every) {
-      const size_t j = snap / snap_every - 1u;
-      if (j >= nsnap) break;
-      const size_t at = (size_t)row * nsnap + j;
-      longlong2 *to = reinterpret_cast<longlong2 *>(R.snap_E) + at * (size_t)s;
-      for (int y = lane; y < acount; y += 32) to[y] = slotE(y);
-      if (lane == 0) R.snap_count[at] = acount;
+    if constexpr (EXT) {
+      if (snap_every == 0u) return;
+      for (; snap <= upto && snap != 0u; snap += snap_every) {
+        const size_t j = snap / snap_every - 1u;
+        if (j >= nsnap) break;
+        const size_t at = (size_t)row * nsnap + j;
+        longlong2 *to = reinterpret_cast<longlong2 *>(R.snap_E) + at * (size_t)s;
+        for (int y = lane; y < acount; y += 32) to[y] = slotE(y);
+        if (lane == 0) R.snap_count[at] = acount;
+      }
     }
   };
 
