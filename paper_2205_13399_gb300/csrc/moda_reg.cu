@@ -45,6 +45,10 @@ int reg_words(int W, bool draws, bool crowded) {
   return W <= 56 ? 4 : W <= 176 ? 8 : W <= 16 * kRegMaxWorkers ? 16 : 24;
 }
 
+// Warps that the registers of a kernel of K words allow in one block: each
+// quarter of an SM holds whole warps only (K = 24: 5 of 96 registers).
+static int reg_most_warps(int K) { return 4 * (16384 / (32 * reg_regs(K))); }
+
 RegFit reg_fit(int n, int64_t fmax, int64_t dmax, int s, bool narrow, bool ext, int optin) {
   const int m = n * n, W = (m + 31) / 32;
   const bool wide = !narrow || ext, draws = narrow || ext;
@@ -52,7 +56,7 @@ RegFit reg_fit(int n, int64_t fmax, int64_t dmax, int s, bool narrow, bool ext, 
   if (fmax > 65535 || dmax > 65535) return RegFit{};
   for (const bool crowded : {false, true}) {
     const int K = reg_words(W, draws, crowded), workers = (W + K - 1) / K;
-    if (workers > kRegMaxWorkers) return RegFit{};
+    if (workers > kRegMaxWorkers || workers + 2 > reg_most_warps(K)) return RegFit{};
     RegFit g;
     for (const bool mma : {2 * dmax <= 65535, false})
       for (int se = std::min(s, kRegSlots); se >= 1 && g.se == 0; se = se > 64 ? se / 2 : se / 8)

@@ -62,6 +62,18 @@ def test_rebuilds_over_the_value_ranges(n, fmax, dmax, replicas):
     assert res.stats[:, 7].sum() > 0  # some jumps rebuilt
 
 
+# the widest tiling ends at 18 workers of 24 words: 432 words, n = 117
+@pytest.mark.parametrize("n", [115, 116, 117, 118, 128])
+@pytest.mark.parametrize("replicas", [2, 160])
+def test_the_largest_sizes(n, replicas):
+    inst = inputs.euclid_instance(n, 0.0, False, index=n, workload="BATCH")
+    kw = dict(I_max=150, seed=n, delta0=2e7, deltaf=3e4, xi=0.05)
+    _, _, res, tr = gpu_run(inst, trace=True, replicas=replicas, **kw)
+    rows = [0, replicas - 1]
+    _, orc = oracle_run(inst, trace=True, replicas=rows, **kw)
+    compare(res, rows, orc, n * n, gpu_trace=tr)
+
+
 @pytest.mark.parametrize("acc", ["strict", "lenient"])
 @pytest.mark.parametrize("n,weights", [(41, None), (57, None), (9, (10 ** 12, 3))])
 def test_delta_e_beyond_int32(n, weights, acc):
