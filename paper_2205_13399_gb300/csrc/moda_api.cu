@@ -621,8 +621,8 @@ moda_status prepare_warp_run(moda_instance inst, const moda_params *p, cudaStrea
   w.s = r->s;
   w.narrow = narrow ? 1 : 0;
   w.se = fit.se;
-  w.mma = fit.mma ? 1 : 0;
-  w.fbig = inst->fmax > 255 ? 1 : 0;
+  w.mma = fit.mma;
+  w.fbig = moda::reg_split_flows(inst->fmax, inst->dmax, inst->n) ? 1 : 0;
   w.dmax = (int32_t)std::min<int64_t>(inst->dmax, 65535);
   w.arch_min = r->arch_min;
   w.hm_limit = moda::reg_hm_limit(inst->b1, inst->b2, inst->w1, inst->w2);

@@ -368,8 +368,9 @@ struct WarpRun {
   // [R][s] or nullptr; largest R_i + C_u at which every Delta E fits int32
   uint32_t *arch_min;
   int32_t hm_limit;
-  int32_t mma;               // rebuilds by matrix products: 2 max d < 2^16 and room
-  int32_t fbig, dmax;        // some Fs entry > 255; largest distance
+  int32_t mma;               // rebuilds by matrix products: 0 no (2 max d >= 2^16, or
+                             // no room), 1 yes, 2 with fp16 planes of Fs
+  int32_t fbig, dmax;        // flows split into bytes for it; largest distance
   // its extensions (ext of the launch): normalisation with its scales, the
   // offset escape, archive snapshots (moda_params)
   int32_t normalize, escape, snap_every, nsnap;
@@ -454,17 +455,33 @@ __host__ __device__ constexpr int reg_regs(int K) {
   return K <= 2 ? 72 : K == 4 ? 64 : K == 8 ? 80 : K == 16 ? 72 : 96;
 }
 
-// Rebuild by matrix products (flag mma of a run): M^T as bytes, one row per
-// column u (padded to tiles of 8), `mstride` bytes a row (k padded to 32,
-// plus 16 so that the eight rows of a fragment fall in different banks).
-__host__ __device__ inline int reg_mstride(int n) { return (n + 31) / 32 * 32 + 16; }
+// Rebuild by matrix products (flag mma of a run): bytes of a row of fp16
+// entries, n padded to 16 of them, plus 16 so that the eight rows of a
+// fragment fall in different banks.
+__host__ __device__ inline int reg_mstride(int n) { return (n + 15) / 16 * 32 + 16; }
+// Whether entries of M up to mmax go in whole: exact in fp16, and their
+// products with a byte summed over n stay below 2^24.
+__host__ __device__ inline bool reg_whole(int mmax, int n) {
+  return mmax <= 2047 && 255 * mmax * n < (1 << 24);
+}
+// Whether flows up to fmax have to be split into bytes, so that the sums with
+// entries of M (one or two distances up to dmax, whole or their bytes) stay
+// below 2^24 and the entries below 1,024.
+inline bool reg_split_flows(int64_t fmax, int64_t dmax, int n) {
+  int64_t cap = 255;  // the largest entry of M or of its bytes
+  for (const int64_t d : {dmax, 2 * dmax})
+    if (d <= 2047 && reg_whole((int)d, n) && d > cap) cap = d;
+  return fmax > 1023 || fmax * cap * n >= (1 << 24);
+}
+
+constexpr int kRegStrip = 32;  // rows of L a rebuild hands over at a time
 
 struct RegSmem {
-  uint32_t fs, d, ring, cnt, min, flip, tgt, jump, rc, v2, x, sum, rcp, draw, scr, mt, aE, aM,
+  uint32_t fs, d, ring, cnt, min, flip, tgt, jump, rc, v2, x, sum, rcp, draw, scr, mt, pl, aE, aM,
       total;
 };
 __host__ __device__ inline RegSmem reg_smem(int n, int m, int se, int workers, int K, bool wide,
-                                            bool inl, bool mma) {
+                                            bool inl, int mma, bool fbig) {
   const int nc = (m + 127) / 128;
   RegSmem L;
   size_t o = 0;
@@ -483,10 +500,12 @@ __host__ __device__ inline RegSmem reg_smem(int n, int m, int se, int workers, i
   L.rcp = (uint32_t)o;   if (wide) o = align_up(o + 2 * (size_t)kMaxN * (size_t)workers, 16);
   // levels: of two iterations, or of one chunk per worker
   L.draw = (uint32_t)o;  o = align_up(o + 512 * (inl ? (size_t)workers : 2 * (size_t)nc), 16);
-  // a strip of 16 rows of (L_1, L_2), or 32 rows of M = X D
-  L.scr = (uint32_t)o;   o = align_up(o + 8 * 16 * (size_t)n, 16);
+  // a strip of (L_1, L_2), or 32 rows of M = X D
+  L.scr = (uint32_t)o;   o = align_up(o + 8 * (size_t)kRegStrip * n, 16);
   L.mt = (uint32_t)o;
-  if (mma) o = align_up(o + 2 * (size_t)((n + 7) / 8 * 8) * reg_mstride(n), 16);
+  if (mma) o = align_up(o + (size_t)((n + 7) / 8 * 8) * reg_mstride(n), 16);
+  L.pl = (uint32_t)o;  // fp16 planes of Fs
+  if (mma == 2) o = align_up(o + (fbig ? 4 : 2) * (size_t)((n + 15) / 16 * 16) * reg_mstride(n), 16);
   // archive slots on chip, and one that only takes stores
   L.aE = (uint32_t)o;    o = align_up(o + 16 * ((size_t)se + 1), 16);
   L.aM = (uint32_t)o;    o = align_up(o + 4 * ((size_t)se + 1), 16);
@@ -514,11 +533,11 @@ int reg_words(int W, bool draws, bool crowded);
 
 // How a run fits the register annealer, at either choice of words per worker
 // (the launch is planned later): its archive slots on chip (0: it cannot run
-// there) and whether rebuilds use matrix products.  Flows are packed as 16
+// there) and how rebuilds use matrix products (WarpRun::mma).  Flows are packed as 16
 // bits, and everything but the slots must fit in shared memory.
 struct RegFit {
   int se = 0;
-  bool mma = false;
+  int mma = 0;
 };
 RegFit reg_fit(int n, int64_t fmax, int64_t dmax, int s, bool narrow, bool ext, int optin);
 
@@ -529,13 +548,14 @@ int32_t reg_hm_limit(int64_t b1, int64_t b2, int64_t w1, int64_t w2);
 
 // The launch shape for `items` replicas of the `count` runs: the fewest words
 // per worker whose blocks are all resident at once, else the choice for a
-// crowded device.  K = 0: no shape fits.
+// crowded device, there without planes of Fs (runs[].mma is lowered) where
+// they would cost resident blocks.  K = 0: no shape fits.
 struct RegChoice {
   int K = 0, workers = 0, draws = 0;
   size_t smem = 0;
   const void *func = nullptr;
 };
-cudaError_t reg_choose(const WarpRun *runs, int count, int64_t items, bool ext, int sms, int optin,
+cudaError_t reg_choose(WarpRun *runs, int count, int64_t items, bool ext, int sms, int optin,
                        RegChoice *out);
 
 // The kernel with K words per worker (1, 2 with draw warps and int32 Delta E

@@ -5,8 +5,10 @@
 // stall every request), or code whose device memory is owned by a host
 // framework that forbids allocations outside its allocator.  This entry
 // point takes the instance from host arrays and writes into device output
-// buffers the caller owns; everything else the kernel needs -- its field
-// cache (scratch), the cooling schedule, the -ln(u) table and the
+// buffers the caller owns; everything else the kernel needs -- its scratch
+// (the block engine's field cache; the register annealer, which runs
+// wherever it holds the run, keeps there the least penalties of the archive
+// slots beyond its shared memory), the cooling schedule, the -ln(u) table and the
 // instance's matrices -- lives in file-scope device arrays of fixed size,
 // which every GPU that loads this library holds until the process exits.
 //
@@ -305,8 +307,8 @@ extern "C" moda_status moda_anneal_noalloc(int32_t n, const int16_t *F1,
       w.W = W;
       w.s = s;
       w.se = fit.se;
-      w.mma = fit.mma ? 1 : 0;
-      w.fbig = std::max(e1max, e2max) > 255 ? 1 : 0;
+      w.mma = fit.mma;
+      w.fbig = moda::reg_split_flows(std::max(e1max, e2max), edmax, n) ? 1 : 0;
       w.dmax = (int32_t)edmax;
       w.arch_min = spill ? reinterpret_cast<uint32_t *>(S->scratch) : nullptr;
       w.hm_limit = moda::reg_hm_limit(f1max * dmax, f2max * dmax, w1, w2);

@@ -45,6 +45,12 @@ int reg_words(int W, bool draws, bool crowded) {
   return W <= 56 ? 4 : W <= 176 ? 8 : W <= 16 * kRegMaxWorkers ? 16 : 24;
 }
 
+// Rebuilds: planes of Fs where no slot has to go for them, then matrix
+// products from the rows, then neither.  Products from n = 29 up: n = 20 (3,000
+// replicas) 81 ms without and 104 with them, n = 25 13.6 and 13.8, n = 33 28.7
+// and 27.8, n = 50 59.1 and 48.6, n = 75 88.1 and 60.2.
+constexpr int kRegMma = 29;
+
 // Warps that the registers of a kernel of K words allow in one block: each
 // quarter of an SM holds whole warps only (K = 24: 5 of 96 registers).
 static int reg_most_warps(int K) { return 4 * (16384 / (32 * reg_regs(K))); }
@@ -52,18 +58,22 @@ static int reg_most_warps(int K) { return 4 * (16384 / (32 * reg_regs(K))); }
 RegFit reg_fit(int n, int64_t fmax, int64_t dmax, int s, bool narrow, bool ext, int optin) {
   const int m = n * n, W = (m + 31) / 32;
   const bool wide = !narrow || ext, draws = narrow || ext;
-  RegFit f{kRegSlots, true};
+  RegFit f{kRegSlots, 2};
   if (fmax > 65535 || dmax > 65535) return RegFit{};
   for (const bool crowded : {false, true}) {
     const int K = reg_words(W, draws, crowded), workers = (W + K - 1) / K;
     if (workers > kRegMaxWorkers || workers + 2 > reg_most_warps(K)) return RegFit{};
     RegFit g;
-    for (const bool mma : {2 * dmax <= 65535, false})
-      for (int se = std::min(s, kRegSlots); se >= 1 && g.se == 0; se = se > 64 ? se / 2 : se / 8)
-        if ((int64_t)reg_smem(n, m, se, workers, K, wide, K >= 4, mma).total <= optin)
+    for (int mma = 2 * dmax <= 65535 && n >= kRegMma ? 2 : 0; mma >= 0 && g.se == 0; --mma)
+      for (int se = std::min(s, kRegSlots); se >= 1 && g.se == 0; se = se > 64 ? se / 2 : se / 8) {
+        if (mma == 2 && se < std::min(s, kRegSlots)) break;
+        if ((int64_t)reg_smem(n, m, se, workers, K, wide, K >= 4, mma,
+                              reg_split_flows(fmax, dmax, n))
+                         .total <= optin)
           g = RegFit{se, mma};
+      }
     f.se = std::min(f.se, g.se);
-    f.mma = f.mma && g.mma;
+    f.mma = std::min(f.mma, g.mma);
   }
   return f;
 }
@@ -76,7 +86,7 @@ int32_t reg_hm_limit(int64_t b1, int64_t b2, int64_t w1, int64_t w2) {
   return (int32_t)std::max<int64_t>(lim, -1);
 }
 
-cudaError_t reg_choose(const WarpRun *runs, int count, int64_t items, bool ext, int sms, int optin,
+cudaError_t reg_choose(WarpRun *runs, int count, int64_t items, bool ext, int sms, int optin,
                        RegChoice *out) {
   *out = RegChoice{};
   int W = 1;
@@ -86,18 +96,28 @@ cudaError_t reg_choose(const WarpRun *runs, int count, int64_t items, bool ext, 
   for (int K = reg_words(W, draws, false); K <= 24; K = K < 8 ? 2 * K : K + 8) {
     const int g = (W + K - 1) / K, d = K < 4 ? std::min((W + 3) / 4, 6) : 0;
     const bool inl = K >= 4;
-    size_t need = 0;
-    for (int k = 0; k < count; ++k)
-      need = std::max<size_t>(need, reg_smem(runs[k].n, runs[k].m, runs[k].se, g, K, wide, inl,
-                                             runs[k].mma != 0)
-                                        .total);
-    if (g > kRegMaxWorkers || need > (size_t)optin) continue;
+    auto need_of = [&](int most) {
+      size_t need = 0;
+      for (int k = 0; k < count; ++k)
+        need = std::max<size_t>(need, reg_smem(runs[k].n, runs[k].m, runs[k].se, g, K, wide, inl,
+                                               std::min(runs[k].mma, most), runs[k].fbig != 0)
+                                          .total);
+      return need;
+    };
+    size_t need = need_of(2);
+    if (g > kRegMaxWorkers || need_of(1) > (size_t)optin) continue;
     const void *func = nullptr;
     cudaError_t e = reg_function(K, narrow, runs[0].accept != 0, ext, optin, &func);
     if (e != cudaSuccess) return e;
-    int blocks = 0;
-    e = reg_occupancy(func, g + d + 2, need, &blocks);
+    int blocks = 0, lean = 0;
+    if (need <= (size_t)optin) e = reg_occupancy(func, g + d + 2, need, &blocks);
+    if (e == cudaSuccess) e = reg_occupancy(func, g + d + 2, need_of(1), &lean);
     if (e != cudaSuccess) return e;
+    if (lean > blocks && (int64_t)blocks * sms < items) {
+      for (int k = 0; k < count; ++k) runs[k].mma = std::min(runs[k].mma, 1);
+      need = need_of(1);
+      blocks = lean;
+    }
     if (blocks >= 1 && ((int64_t)blocks * sms >= items || K >= crowded)) {
       *out = RegChoice{K, g, d, need, func};
       return cudaSuccess;

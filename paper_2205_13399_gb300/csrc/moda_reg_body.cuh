@@ -47,8 +47,11 @@
 // (of 1,072 on n = 75, all), and that a run has about 1,000 of them.
 //
 // Rebuilds.  L_k = Fs_k M with M = X D is a contraction of three n x n
-// matrices; with at most two bits a row M fits 16 bits, so it runs on the
-// tensor cores exactly: bytes of Fs_k times bytes of M, 32-bit sums.
+// matrices, and with at most two bits a row it runs on the tensor cores
+// exactly: fp16 holds integers up to 2,048, so entries of Fs_k and M (or
+// their bytes, where a sum could pass 2^24) are multiplied and summed in
+// float without rounding.  (The 8-bit integer form of the same instruction
+// is slow on this part: a strip of 16 rows took 3,700 cycles on n = 75.)
 #pragma once
 
 #include <cstdint>
@@ -85,13 +88,26 @@ static_assert(sizeof(RFlip) == 24, "flip record layout");
 __device__ __forceinline__ int uni(int v) { return __shfl_sync(kFull, v, 0); }
 __device__ __forceinline__ uint32_t uni(uint32_t v) { return __shfl_sync(kFull, v, 0); }
 
-// D (16 x 8, int32) += A (16 x 32 bytes, rows) B (32 x 8 bytes, columns).
-__device__ __forceinline__ void mma_u8(int32_t (&d)[4], const uint32_t (&a)[4], uint32_t b0,
-                                       uint32_t b1) {
-  asm("mma.sync.aligned.m16n8k32.row.col.s32.u8.u8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+// D (16 x 8, float) += A (16 x 16 fp16, rows) B (16 x 8 fp16, columns).
+__device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
+                                        uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
       "{%8, %9}, {%0, %1, %2, %3};"
-      : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// fp16 of an integer up to 2,048 (exact), in the low half
+__device__ __forceinline__ uint32_t half_of(uint32_t v) {
+  uint16_t h;
+  asm("cvt.rn.f16.u16 %0, %1;" : "=h"(h) : "h"((uint16_t)v));
+  return h;
+}
+// fp16 pair of two integers below 1,024 in the halves of x: 1,024 + v has v in
+// its mantissa, less 1,024
+__device__ __forceinline__ uint32_t halves_of(uint32_t x) {
+  uint32_t r;
+  asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(x | 0x64006400u), "r"(0xE400E400u));
+  return r;
 }
 
 // EXT carries the options beyond the default algorithm, chosen at run time:
@@ -128,7 +144,8 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   const uint32_t magic = uni(R.magic);
   const double *const table = R.table;
   const int hm_limit = uni(R.hm_limit);
-  const bool use_mma = uni(R.mma) != 0, fbig = uni(R.fbig) != 0;
+  const int use_mma = uni(R.mma);  // 1: fragments from the flow rows, 2: from fp16 planes of Fs
+  const bool fbig = uni(R.fbig) != 0;
   const int dmax = uni(R.dmax);
   auto divn = [&](int p) { return (int)__umulhi((uint32_t)p, magic); };
   const bool lenient = EXT ? uni(R.accept) != 0 : LEN;
@@ -146,7 +163,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     return hi < 0xFFFFFFFFll ? (uint32_t)hi : 0xFFFFFFFFu;
   };
 
-  const RegSmem SL = reg_smem(n, m, se, G, K, WIDE, INL, use_mma);
+  const RegSmem SL = reg_smem(n, m, se, G, K, WIDE, INL, use_mma, fbig);
   constexpr int kFb = F64 ? 8 : 4;       // bytes of a flow pair
   const int fcols = reg_fcols(n, F64);
   const int frow = fcols * kFb;          // bytes of a flow row: n pairs and zeros
@@ -345,20 +362,46 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     if (lane == 0) *sHm = a + b;
   };
 
+  if (use_mma == 2) {
+    // Fs as fp16 for the rebuilds, zero past n: one plane an objective, or
+    // (fbig) its low and its high bytes
+    const int ms = reg_mstride(n), rows = (n + 15) / 16 * 16;
+    for (int e = threadIdx.x; e < rows * (ms / 4); e += threads) {
+      const int i = e / (ms / 4), j = 2 * (e - i * (ms / 4));
+      uint32_t b[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+        if (i < n && j + q < n) {
+          const uint32_t f1 = (uint32_t)R.Fs1[i * n + j + q], f2 = (uint32_t)R.Fs2[i * n + j + q];
+          b[0] |= half_of(fbig ? f1 & 255u : f1) << (16 * q);
+          b[1] |= half_of(f1 >> 8) << (16 * q);
+          b[2] |= half_of(fbig ? f2 & 255u : f2) << (16 * q);
+          b[3] |= half_of(f2 >> 8) << (16 * q);
+        }
+#pragma unroll
+      for (int f = 0; f < 4; ++f)
+        if (fbig || f % 2 == 0)
+          *reinterpret_cast<uint32_t *>(smem + SL.pl +
+                                        (size_t)(fbig ? f : f / 2) * rows * ms + 4 * e) = b[f];
+    }
+  }
+
   // Delta E of the state in sX from scratch (Alg. 3's initial state, or the
   // member a jump landed on), by the whole block: the counts, then
   // L_k(i,u) = sum_j Fs^k_ij M_ju with M = X D, by matrix products where the
   // rows have at most two bits, else from blocks of rows of M in shared
   // memory.  Starts with a block barrier after which sX must be complete and
   // ends on one.  energies: also sums over the set bits of L_1 and L_2
-  // (2 c_k) per warp into sSum.
-  auto rebuild = [&](bool energies) {
+  // (2 c_k) per warp into sSum.  aside(): what the last (store) warp does while
+  // the others scatter the set bits and form M.
+  auto rebuild = [&](bool energies, auto &&aside) {
+    const bool helps = wid != warps - 1;
     for (int i = threadIdx.x; i < 2 * kMaxN; i += threads) sR[i] = 0;
     for (int i = threadIdx.x; i < kMaxN / 2; i += threads)
       reinterpret_cast<uint32_t *>(sV)[i] = 0xFFFFFFFFu;
     if (threadIdx.x == 0) *sFlags = 0u;
     __syncthreads();
-    for (int w = threadIdx.x; w < W; w += threads) {
+    for (int w = threadIdx.x; helps && w < W; w += threads - 32) {
       uint32_t v = sX[w];
       while (v) {
         const int p = 32 * w + __ffs(v) - 1;
@@ -370,118 +413,144 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
         if (had >= 1) atomicOr(sFlags, had == 1 ? 1u : 2u);
       }
     }
+    if (!helps) aside();
     xn = 0u;
 #pragma unroll
     for (int k = 0; k < K; ++k)
       if (w0 + k < W) xn |= ((sX[w0 + k] >> lane) & 1u) << k;
     __syncthreads();
     const uint32_t flags = uni(*reinterpret_cast<volatile uint32_t *>(sFlags));
-    if (use_mma && (flags & 2u) == 0u) {
-      // ---- M^T in bytes: row u, column j holds sum_v x_jv d_uv (two planes
-      // when an entry may pass 255)
-      const int ms = reg_mstride(n), mu = (n + 7) / 8 * 8, kq = (n + 31) / 32 * 8;
-      unsigned char *const mlo = smem + SL.mt, *const mhi = mlo + (size_t)mu * ms;
-      const bool mbig = dmax > 255 || ((flags & 1u) && 2 * dmax > 255);
+    if (use_mma != 0 && (flags & 2u) == 0u) {
+      const int ms = reg_mstride(n), kq = (n + 15) / 16 * 4;
+      unsigned char *const mt = smem + SL.mt;
       const int32_t *const dd = reinterpret_cast<const int32_t *>(sD);
-      for (int jq = lane; jq < kq; jq += 32) {
-        uint32_t vv[4];  // two columns of each of the four rows 4 jq ..
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          vv[q] = 4 * jq + q < n ? reinterpret_cast<const uint16_t *>(sV)[4 * jq + q] : 0xFFFFu;
-        for (int u = wid; u < n; u += warps) {
-          uint32_t lo = 0u, hi = 0u;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const uint32_t a = vv[q] & 255u, b = vv[q] >> 8;
-            uint32_t mm = 0u;
-            if (a != 255u) mm = (uint32_t)dd[a * n + u];
-            if (b != 255u) mm += (uint32_t)dd[b * n + u];
-            lo |= (mm & 255u) << (8 * q);
-            hi |= (mm >> 8) << (8 * q);
-          }
-          *reinterpret_cast<uint32_t *>(mlo + u * ms + 4 * jq) = lo;
-          if (mbig) *reinterpret_cast<uint32_t *>(mhi + u * ms + 4 * jq) = hi;
-        }
-      }
-      __syncthreads();
-      // ---- strips of 16 rows: every warp takes tiles of 8 columns; A is
-      // Fs (symmetric: flow row j, split into bytes by permutes; the stride
-      // of a flow row keeps a fragment's loads free of bank conflicts, which
-      // were 4-way without it), the products of byte planes add up shifted
-      // by their weights
+      // one pass with whole entries of M where every sum of products stays
+      // below 2^24 (the host chose fbig for the same), else one per byte
+      const int mmax = (flags & 1u) ? 2 * dmax : dmax;
+      const bool whole = reg_whole(mmax, n);
       int2 *const sL = reinterpret_cast<int2 *>(smem + SL.scr);
-      const int gi = lane >> 2, ti = lane & 3;
-      for (int ib = 0; ib < n; ib += 16) {
-        for (int ut = 8 * wid; ut < n; ut += 8 * warps) {
-          uint32_t l1[4] = {0u, 0u, 0u, 0u}, l2[4] = {0u, 0u, 0u, 0u};
-#pragma unroll 1
-          for (int mp = 0; mp <= (mbig ? 1 : 0); ++mp) {  // the byte of M
-            const unsigned char *bm = (mp ? mhi : mlo) + (ut + gi) * ms + 4 * ti;
-            int32_t c[4][4];
+      const int gi = lane >> 2, ti = lane & 3, ut8 = (n + 7) / 8;
+      const int prow = (n + 15) / 16 * 16;  // rows of a plane of Fs
+      for (int mp = 0; mp < (whole ? 1 : 2); ++mp) {
+        // ---- M^T as fp16: row u, column j holds sum_v x_jv d_uv (or its
+        // byte mp)
+        for (int jq = lane; helps && jq < kq; jq += 32) {
+          uint32_t vv[4];  // two columns of each of the four rows 4 jq ..
 #pragma unroll
-            for (int f = 0; f < 4; ++f) c[f][0] = c[f][1] = c[f][2] = c[f][3] = 0;
+          for (int q = 0; q < 4; ++q)
+            vv[q] = 4 * jq + q < n ? reinterpret_cast<const uint16_t *>(sV)[4 * jq + q] : 0xFFFFu;
+          for (int u = wid; u < n; u += warps - 1) {
+            uint32_t h[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const uint32_t a = vv[q] & 255u, b = vv[q] >> 8;
+              uint32_t mm = 0u;
+              if (a != 255u) mm = (uint32_t)dd[a * n + u];
+              if (b != 255u) mm += (uint32_t)dd[b * n + u];
+              h[q] = half_of(whole ? mm : (mm >> (8 * mp)) & 255u);
+            }
+            *reinterpret_cast<uint2 *>(mt + u * ms + 8 * jq) =
+                make_uint2(h[0] | h[1] << 16, h[2] | h[3] << 16);
+          }
+        }
+        __syncthreads();
+        // ---- strips of 32 rows, tiles of 16 rows by 8 columns shared out
+        // over the warps.  A is Fs (symmetric: flow row j), from its planes
+        // where they fit (a fragment register is one load), else formed from
+        // the rows (whose stride keeps the loads free of bank conflicts).
+        // Where there are more tiles than warps (n = 50) a warp takes both
+        // halves of its columns at once, in the accumulators of the high
+        // bytes: 51.4 -> 48.5 ms there, 8 words a worker.
+        for (int is = 0; is < n; is += kRegStrip) {
+          const int parts = is + 16 < n ? 2 : 1;  // halves of the strip with rows below n
+          const bool both = K == 8 && use_mma == 2 && !fbig && parts == 2 && 2 * ut8 > warps;
+          const int odd = both ? 16 * ms : prow * ms;
+          for (int job = wid; job < (both ? 1 : parts) * ut8; job += warps) {
+            const int half = job >= ut8 ? 1 : 0;
+            const int ib = is + 16 * half, ut = 8 * (job - half * ut8);
+            const unsigned char *const bm = mt + (ut + gi) * ms + 4 * ti;
+            float c[4][4];  // [objective, low and high bytes of Fs or halves]
+#pragma unroll
+            for (int f = 0; f < 4; ++f) c[f][0] = c[f][1] = c[f][2] = c[f][3] = 0.f;
 #pragma unroll 1
-            for (int kb = 0; kb < n; kb += 32) {
+            for (int kb = 0; kb < n; kb += 16) {
               uint32_t a[4][4];  // [plane][fragment register]
+              if (use_mma == 2) {
+                const unsigned char *ap = smem + SL.pl + (ib + gi) * ms + 2 * kb + 4 * ti;
 #pragma unroll
-              for (int h = 0; h < 4; ++h) {
-                const int i = min(ib + gi + 8 * (h & 1), n - 1);
-                const int j = kb + 4 * ti + 16 * (h >> 1);
-                uint32_t w[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                  const unsigned char *fp = sFs + min(j + q, n - 1) * frow + i * kFb;
-                  if (F64) {
-                    const uint2 f = *reinterpret_cast<const uint2 *>(fp);
-                    w[q] = __byte_perm(f.x, f.y, 0x5410);
-                  } else {
-                    w[q] = *reinterpret_cast<const uint32_t *>(fp);
+                for (int h = 0; h < 4; ++h) {
+                  const int o = 8 * (h & 1) * ms + 16 * (h >> 1);
+                  a[0][h] = *reinterpret_cast<const uint32_t *>(ap + o);
+                  a[2][h] = *reinterpret_cast<const uint32_t *>(ap + o + (fbig ? 2 : 1) * prow * ms);
+                  if (fbig || both) {
+                    a[1][h] = *reinterpret_cast<const uint32_t *>(ap + o + odd);
+                    a[3][h] = *reinterpret_cast<const uint32_t *>(
+                        ap + o + odd + (fbig ? 2 : 1) * prow * ms);
                   }
                 }
-                const uint32_t t0 = __byte_perm(w[0], w[1], 0x5140),
-                               t1 = __byte_perm(w[2], w[3], 0x5140),
-                               t2 = __byte_perm(w[0], w[1], 0x7362),
-                               t3 = __byte_perm(w[2], w[3], 0x7362);
-                a[0][h] = __byte_perm(t0, t1, 0x5410);
-                a[1][h] = __byte_perm(t0, t1, 0x7632);
-                a[2][h] = __byte_perm(t2, t3, 0x5410);
-                a[3][h] = __byte_perm(t2, t3, 0x7632);
+              } else {
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                  const int i = min(ib + gi + 8 * (h & 1), n - 1);
+                  const int j = kb + 2 * ti + 8 * (h >> 1);
+                  uint32_t w[2];
+#pragma unroll
+                  for (int q = 0; q < 2; ++q) {
+                    const unsigned char *fp = sFs + min(j + q, n - 1) * frow + i * kFb;
+                    if (F64) {
+                      const uint2 f = *reinterpret_cast<const uint2 *>(fp);
+                      w[q] = __byte_perm(f.x, f.y, 0x5410);
+                    } else {
+                      w[q] = *reinterpret_cast<const uint32_t *>(fp);
+                    }
+                  }
+                  const uint32_t x1 = __byte_perm(w[0], w[1], 0x5410),
+                                 x2 = __byte_perm(w[0], w[1], 0x7632);
+                  a[0][h] = halves_of(fbig ? x1 & 0x00FF00FFu : x1);
+                  a[2][h] = halves_of(fbig ? x2 & 0x00FF00FFu : x2);
+                  a[1][h] = fbig ? halves_of((x1 >> 8) & 0x00FF00FFu) : 0u;
+                  a[3][h] = fbig ? halves_of((x2 >> 8) & 0x00FF00FFu) : 0u;
+                }
               }
-              const uint32_t b0 = *reinterpret_cast<const uint32_t *>(bm + kb);
-              const uint32_t b1 = *reinterpret_cast<const uint32_t *>(bm + kb + 16);
-              mma_u8(c[0], a[0], b0, b1);
-              mma_u8(c[2], a[2], b0, b1);
-              if (fbig) {
-                mma_u8(c[1], a[1], b0, b1);
-                mma_u8(c[3], a[3], b0, b1);
+              const uint32_t b0 = *reinterpret_cast<const uint32_t *>(bm + 2 * kb);
+              const uint32_t b1 = *reinterpret_cast<const uint32_t *>(bm + 2 * kb + 16);
+              mma_f16(c[0], a[0], b0, b1);
+              mma_f16(c[2], a[2], b0, b1);
+              if (fbig || both) {
+                mma_f16(c[1], a[1], b0, b1);
+                mma_f16(c[3], a[3], b0, b1);
               }
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-              l1[q] += ((uint32_t)c[0][q] + ((uint32_t)c[1][q] << 8)) << (8 * mp);
-              l2[q] += ((uint32_t)c[2][q] + ((uint32_t)c[3][q] << 8)) << (8 * mp);
+              uint32_t v[4];
+#pragma unroll
+              for (int f = 0; f < 4; ++f) v[f] = __float2uint_rn(c[f][q]);
+              const int r = 16 * half + gi + 8 * (q >> 1), u = ut + 2 * ti + (q & 1);
+              if (u < n) {
+                const uint32_t h1 = both ? 0u : v[1] << 8, h2 = both ? 0u : v[3] << 8;
+                sL[r * n + u] =
+                    make_int2((int)((v[0] + h1) << (8 * mp)), (int)((v[2] + h2) << (8 * mp)));
+                if (both)
+                  sL[(r + 16) * n + u] = make_int2((int)(v[1] << (8 * mp)), (int)(v[3] << (8 * mp)));
+              }
             }
           }
+          __syncthreads();
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int r = gi + 8 * (q >> 1), u = ut + 2 * ti + (q & 1);
-            if (u < n) sL[r * n + u] = make_int2((int)l1[q], (int)l2[q]);
-          }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-          const int p = 32 * (w0 + k);
-          if (p < (ib + 16) * n && p + 32 > ib * n) {
-            const int i = i_of(k) - ib;
-            if (i >= 0 && i < 16 && i + ib < n) {
-              const int2 v = sL[i * n + u_of(k)];
-              e1[k] = (uint32_t)v.x;
-              e2[k] = (uint32_t)v.y;
+          for (int k = 0; k < K; ++k) {
+            const int p = 32 * (w0 + k);
+            if (p < (is + kRegStrip) * n && p + 32 > is * n) {
+              const int i = i_of(k) - is;
+              if (i >= 0 && i < kRegStrip && i + is < n) {
+                const int2 v = sL[i * n + u_of(k)];
+                e1[k] = (uint32_t)v.x + (mp ? e1[k] : 0u);
+                e2[k] = (uint32_t)v.y + (mp ? e2[k] : 0u);
+              }
             }
           }
+          __syncthreads();
         }
-        __syncthreads();
       }
     } else {
       int32_t *const sM = reinterpret_cast<int32_t *>(smem + SL.scr);
@@ -583,7 +652,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   };
 
   __syncthreads();
-  rebuild(true);
+  rebuild(true, [] {});
 
   if (wid >= G && wid < G + D) {
     // ================= draw warps =================
@@ -608,7 +677,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
         const uint32_t mode = uni(sJ[0]);
         t = uni(sJ[1]);
         if (mode == kRegEnd || mode == kRegStayEnd) break;
-        if (mode == kRegRebuild) rebuild(false);
+        if (mode == kRegRebuild) rebuild(false, [] {});
         draw(t);
         draw(t + 1u);
         __syncthreads();
@@ -805,7 +874,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
         const uint32_t mode = uni(sJ[0]);
         t = uni(sJ[1]);
         if (mode == kRegEnd || mode == kRegStayEnd) break;
-        if (mode == kRegRebuild) rebuild(false);
+        if (mode == kRegRebuild) rebuild(false, [] {});
         if (D > 0) __syncthreads();  // draws
         trial(t);
         continue;
@@ -992,8 +1061,8 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       if (mode == kRegEnd || mode == kRegRebuild)  // the member the jumps ended on
         for (int q = lane; q < W; q += 32) sX[q] = gB[(size_t)slot * W + q];  // (written here)
       if (mode == kRegEnd || mode == kRegStayEnd) break;
-      refill(t);
-      if (mode == kRegRebuild) rebuild(false);
+      if (mode == kRegRebuild) rebuild(false, [&] { refill(t); });
+      else refill(t);
       if (D > 0) __syncthreads();  // draws
     }
     __syncwarp();
@@ -1272,7 +1341,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     __syncthreads();
     if (end) break;
     ++nrebuild;
-    rebuild(false);
+    rebuild(false, [] {});
     if (D > 0) __syncthreads();  // draws
   }
 

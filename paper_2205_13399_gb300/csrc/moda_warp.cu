@@ -1,6 +1,9 @@
-// The warp annealer: Alg. 3 of arXiv 2205.13399 (the multi-objective
-// Digital Annealer, Sec. 3.3) for the bi-objective QAP with a team of G
-// warps (G = 1 .. 8) per replica.  A persistent grid of teams pulls (run,
+// The team annealer of the warp engine: Alg. 3 of arXiv 2205.13399 (the
+// multi-objective Digital Annealer, Sec. 3.3) for the bi-objective QAP with a
+// team of G warps (G = 1 .. 8) per replica.  It runs the requests that
+// prescribe its layout (team size, prefetch distance, field cache) or that the
+// register annealer does not hold; the others run there, several times faster
+// (moda_reg_body.cuh).  A persistent grid of teams pulls (run,
 // replica) work items from a device list (largest runs first), so replicas
 // of many instances of uneven n share the GPU in one launch; a team
 // synchronises on a named barrier of its own, never on a block barrier.

@@ -62,6 +62,31 @@ def test_rebuilds_over_the_value_ranges(n, fmax, dmax, replicas):
     assert res.stats[:, 7].sum() > 0  # some jumps rebuilt
 
 
+# products from n = 29 up; a last block of 16 rows that is full, ragged or one
+# row (n = 50, where a warp takes both halves of a strip, runs whole in
+# test_gpu_warp.py)
+@pytest.mark.parametrize("n,fmax,dmax", [
+    (28, 99, 120), (29, 99, 120), (32, 99, 1023),   # whole entries of both
+    (33, 400, 119),                                 # flows beyond a byte, whole
+    (33, 900, 119), (33, 9000, 40),                 # flows in two bytes
+    (33, 99, 1024),                                 # M in two bytes
+    (29, 200, 32767), (32, 2000, 1500),             # 2 max d = 65,534; both in bytes
+])
+@pytest.mark.parametrize("replicas", [3, 320])
+def test_matrix_products_over_the_value_ranges(n, fmax, dmax, replicas):
+    rng = np.random.default_rng(n + fmax + dmax)
+    F1, F2 = (rng.integers(0, fmax + 1, (n, n)) * (rng.random((n, n)) < 0.3) for _ in range(2))
+    inst = _Inst(F1, F2, rng.integers(dmax // 2, dmax + 1, (n, n)))
+    w = int((inst.F1.astype(int) + inst.F1.T).sum(1).max()) * int(inst.D.astype(int).sum(1).max())
+    kw = dict(I_max=1500, seed=5, delta0=2.0 * w, deltaf=w / 500.0, xi=0.01)
+    _, _, res, tr = gpu_run(inst, trace=True, replicas=replicas, **kw)
+    rows = [0, replicas - 1]
+    _, orc = oracle_run(inst, trace=True, replicas=rows, **kw)
+    compare(res, rows, orc, n * n, gpu_trace=tr)
+    # three replicas may have no jump to a member that accepts
+    assert replicas == 3 or res.stats[:, 7].sum() > 0
+
+
 # the widest tiling ends at 18 workers of 24 words: 432 words, n = 117
 @pytest.mark.parametrize("n", [115, 116, 117, 118, 128])
 @pytest.mark.parametrize("replicas", [2, 160])
