@@ -47,12 +47,12 @@ L2_FLUSH_BYTES = 512 << 20
 KERNEL_FILES = {
     "anneal_kernel": ("moda_kernel_body.cuh", "moda_kernel.cu", "moda_kernel_special.cu",
                       "moda_internal.h"),
-    "warp_anneal_kernel": ("moda_warp.cu", "moda_device.cuh", "moda_internal.h"),
+    "reg_anneal_kernel": ("moda_reg_body.cuh", "moda_reg.cu", "moda_device.cuh",
+                          "moda_internal.h"),
 }
 KERNEL_TRAFFIC = {
     "anneal_kernel": {"workload": "P25", "bytes": None, "sha256": None},
-    "warp_anneal_kernel": {"workload": "P25", "bytes": 1052635392 + 1924999424,
-                           "sha256": "53a5ceb321a40b0fe68edded14958ce48972a2441468e5ad548d69a129d1f59b"},
+    "reg_anneal_kernel": {"workload": "P25", "bytes": None, "sha256": None},
 }
 
 
@@ -104,7 +104,7 @@ def parse_args(argv=None):
     ap.add_argument("--batch-seq-instances", type=int, default=512,
                     help="default run: BATCH instances also run one after another")
     ap.add_argument("--engine", default="auto", choices=["auto", "block", "warp"],
-                    help="one thread block or one warp per replica (auto: warp when possible)")
+                    help="block engine, or warp engine (auto: warp when possible)")
     ap.add_argument("--autotune", action="store_true",
                     help="pick block shape and prefetch distance by timed trials first")
     ap.add_argument("--no-autotune", action="store_true",
@@ -371,7 +371,7 @@ def batch_measure(args, steps: int, warmup: int, seq_instances: int):
     roofline = roofline_line(ops, statistics.mean(ms) / 1e3, props.multi_processor_count,
                              clk.get("sm_max_mhz") or 2070.0,
                              f"{OPS_PER_BIT_TRIAL} int32 lane-ops per bit-trial")
-    roofline["kernel"] = "warp_anneal_kernel" if args.engine != "block" else "anneal_kernel"
+    roofline["kernel"] = "reg_anneal_kernel" if args.engine != "block" else "anneal_kernel"
     ns = [q.n for q in qis]
     return {
         "metric": "replica-steps/s", "value": value, "unit": "replica-steps/s", "n_gpus": 1,
@@ -610,7 +610,7 @@ def run_sbda(args):
         hi = (max(p[0] for p in allp), max(p[1] for p in allp))
         sb, md = statistics.mean(s_ms), statistics.mean(m_ms)
         return {"normalised": normalize, "sbda_ms": sb, "mda_ms": md,
-                "sbda_over_mda_time": sb / md, "mda_engine": "block" if normalize else "warp",
+                "sbda_over_mda_time": sb / md, "mda_engine": "warp",
                 "sbda_front_points": len(fs), "mda_front_points": len(front_m),
                 "hv_sbda": hv_norm(fs, lo, hi), "hv_mda": hv_norm(front_m, lo, hi)}
 
@@ -667,14 +667,9 @@ def run_hvtrace(args):
         out[acc] = [[(p["c1"], p["c2"]) for p in r.read_archive(snapshot=j, perms=False)
                      if p["feasible"]] for j in range(I_max // K)]
         r.close()
-    # the snapshot cost against the same engine without snapshots (the
-    # block engine: snapshots are one of its options), and the warp engine
-    # a run without snapshots takes by default
-    plain = moda.anneal(inst, replicas=R, I_max=I_max, seed=run["seed"], engine="block").wait()
-    plain_ms = plain.elapsed_ms()
-    plain.close()
+    # the snapshot cost against the same kernel without snapshots
     plain = moda.anneal(inst, replicas=R, I_max=I_max, seed=run["seed"]).wait()
-    warp_ms = plain.elapsed_ms()
+    plain_ms = plain.elapsed_ms()
     plain.close()
     clk = clocks.stop()
     allp = [p for acc in out for f in out[acc] for p in f]
@@ -701,8 +696,7 @@ def run_hvtrace(args):
         "iterations_to_95pct_hv": {acc: reach(hv[acc]) for acc in hv},
         "hv_every_10_snapshots": {acc: [round(v, 4) for v in hv[acc][9::10]] for acc in hv},
         "snapshot_overhead": {"ms_with": ms["strict"], "ms_plain": plain_ms,
-                              "engine": "block",
-                              "ms_default_engine_without_snapshots": warp_ms},
+                              "engine": "warp"},
         "gpu_launches": 2, "clocks": clk,
     }
     print(json.dumps(line), flush=True)
@@ -876,7 +870,7 @@ def main(argv=None):
     roofline = roofline_line(ops_per_launch, statistics.mean(kernel_ms) / 1e3,
                              props.multi_processor_count, sm_max_mhz,
                              f"{OPS_PER_BIT_TRIAL} int32 lane-ops per bit-trial")
-    roofline["kernel"] = "anneal_kernel" if args.engine == "block" else "warp_anneal_kernel"
+    roofline["kernel"] = "anneal_kernel" if args.engine == "block" else "reg_anneal_kernel"
     roofline["traffic"] = kernel_traffic(
         roofline["kernel"], args.workload, I_max, inputs.WORKLOAD_RUN[args.workload]["I_max"])
     if roofline["traffic"] is not None:

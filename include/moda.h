@@ -106,7 +106,9 @@ typedef struct {
                             fields from a per-slot device copy instead of
                             rebuilding them: 0 auto (when it fits in 60 % of
                             free device memory), 1 on (MODA_EUNSUPPORTED if it
-                            does not fit), 2 off.  Results are identical. */
+                            does not fit), 2 off.  Results are identical.  The
+                            register annealer (see `engine`) has no field
+                            cache: 0 and 2 are the same to it. */
   int32_t prefetch;      /* field-cache prefetch distance: 0 auto, k in 1..4
                             (block engine; 1..15 for the warp engine, see
                             `engine`) copies a jump's target k - 1
@@ -144,11 +146,20 @@ typedef struct {
                             identical:
                             1 block: one thread block per replica (all
                               options; lowest latency per iteration);
-                            2 warp: one warp per replica, replicas of many
-                              runs pulled from one device work list (the
-                              archive escape only, without normalize,
-                              snapshot_every or fast_forward;
-                              MODA_EUNSUPPORTED otherwise).  Its field cache
+                            2 warp: replicas of many runs pulled from one
+                              device work list (the archive escape only,
+                              without normalize, snapshot_every or
+                              fast_forward; MODA_EUNSUPPORTED otherwise).
+                              Two kernels serve it.  The register annealer
+                              (one block per replica, Delta E in registers,
+                              jumps settled by the least acceptance penalty
+                              kept per archive slot, no field cache) runs
+                              every request that prescribes none of
+                              prefetch, block_threads, field_cache = 1 and
+                              cache_slots and whose sizes it holds (n <=
+                              117, entries of Fs and D <= 65,535); the
+                              team annealer runs the others, and the rest of
+                              this paragraph is about it.  Its field cache
                               holds the records of the first cache_slots
                               archive slots per resident team (field_cache
                               = 1: all s slots; 2: none); a jump to a slot
@@ -166,9 +177,12 @@ typedef struct {
                               every iteration is still tested; the first
                               iteration that accepts a bit flips and later
                               trials are discarded).
-                            0 auto: warp when the options allow it and
-                              block_threads is 0, else block. */
-  int32_t cache_slots;   /* warp engine, field_cache = 0: archive slots with
+                            0 auto: as 2 when the options allow it and
+                              block_threads is 0; the register annealer also
+                              for the offset escape, normalize and
+                              snapshot_every under the same conditions;
+                              else block. */
+  int32_t cache_slots;   /* team annealer of the warp engine, field_cache = 0: archive slots with
                             field-cache records per team; 0: min(s, 1024),
                             k > 0: min(s, k), fewer where the launch's caches
                             would not fit the memory budget.  A jump to a
@@ -244,7 +258,8 @@ moda_status moda_wait(moda_run run, int64_t timeout_ms);
  *                       jumps that read the record directly, iterations
  *                       settled without being executed (params.fast_forward),
  *                       and jumps that rebuilt the fields of a slot without
- *                       records (warp engine; 0 in the block engine)
+ *                       records (0 in the block engine; in the register
+ *                       annealer every jump whose landing accepts a bit)
  * Any pointer may be NULL.  MODA_EBUSY while the run executes. */
 moda_status moda_read_replica(moda_run run, int32_t r, int32_t *count,
                               int64_t *E, uint32_t *bits, uint32_t *x,
@@ -344,9 +359,11 @@ void moda_qrun_destroy(moda_qrun run);
  * prefetch distances 1 and 2 besides the automatic choice, on `inst` with
  * `params` (trial_iters iterations at the cold end of the schedule, delta =
  * deltaf, on at most one replica per SM); for the warp engine, prefetch
- * distances 0, 2, 6, 10 and 14 on the request's own replicas.  Writes into
- * *best a copy of *params with the fastest block_threads and prefetch; *best_ms (if not NULL) receives the
- * winning trial's time.  Results of a run do not depend on these two
+ * distances 0, 2, 6, 10 and 14 of the team annealer on the request's own
+ * replicas and, where the engine is left open and no layout is prescribed,
+ * the register annealer (prefetch 0).  Writes into *best a copy of *params
+ * with the fastest block_threads and prefetch; *best_ms (if not NULL)
+ * receives the winning trial's time.  Results of a run do not depend on these two
  * fields, so tuning never changes what an anneal computes.  Blocks the
  * calling thread while the trials run on cuda_stream. */
 moda_status moda_autotune(moda_instance inst, const moda_params *params, int32_t trial_iters,
@@ -400,7 +417,8 @@ const char *moda_last_error(void);
  * memory belongs to a host framework's allocator -- so cudaMalloc (and any
  * routine that allocates, torch's included) is off limits to them.
  *
- * moda_anneal_noalloc runs the same kernel as moda_anneal on the same
+ * moda_anneal_noalloc runs the kernels of moda_anneal (the register
+ * annealer where it holds the run, else the block engine) on the same
  * inputs and gives the same results, but allocates nothing: the instance
  * comes from host arrays (as in moda_create_instance), the results go to
  * device buffers the caller owns (below), and the kernel's scratch (the
