@@ -157,7 +157,8 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   const uint32_t snap_every = EXT ? uni((uint32_t)R.snap_every) : 0u;
   const size_t nsnap = EXT ? (size_t)R.nsnap : 0;
   // a value no penalty that any draw accepts passes: floor(delta T_max), at
-  // most 2^32 - 1; EXT: the bits of a float above fl(delta T_max)
+  // most 2^32 - 1; EXT: the bits of a float that the float form of such a
+  // penalty does not pass while E_off = 0 (a trial adds 1e-6 E_off)
   auto top = [&](double delta, int64_t hi) -> uint32_t {
     if (EXT) return __float_as_uint((float)__dmul_rn(delta, __ldg(&table[0])) * (1.f + 2e-6f));
     return hi < 0xFFFFFFFFll ? (uint32_t)hi : 0xFFFFFFFFu;
@@ -330,8 +331,11 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   // EXT: the penalty sum_k (min_k) max(0, s_k Delta E_k - E_off) in float.
   // Near a draw's level each term is at most E_off + 11.8 delta, and its
   // error at most 6 2^-24 of that (Delta E 3, s_k and the product 2, E_off
-  // 1), so two terms are within 7.2e-7 (E_off + 11.8 delta); the margin adds
-  // 1e-6 (E_off + 12 delta).
+  // 1), so two terms are within 7.2e-7 (E_off + 11.8 delta) = 7.2e-7 E_off +
+  // 8.5e-6 delta.  The margin of the test adds 1e-6 (E_off + 12 delta).  The
+  // bound above which a chunk is left out without its draws is (1 + 2e-6)
+  // delta T_max (2.3e-5 delta) and 1e-6 E_off above delta T_max: E_off has no
+  // bound in terms of delta, and its rounding alone can exceed delta T_max.
   auto ext_penalty = [&](int k, bool nar, float off) -> float {
     float f1, f2;
     if (nar) {
@@ -756,7 +760,8 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
         }
       };
       if (INL) {
-        const uint32_t hi = r.hi;
+        const uint32_t hi =
+            EXT ? __float_as_uint(__uint_as_float(r.hi) + 1e-6f * off) : r.hi;
         float *const mine = sDraw + 128 * wid;  // the chunk's levels by bit
 #pragma unroll
         for (int kc = 0; kc < K; kc += 4) {
