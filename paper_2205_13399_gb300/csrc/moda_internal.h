@@ -588,6 +588,37 @@ cudaError_t launch_front(const int32_t *counts, const int64_t *E, int s, int ns,
 cudaError_t launch_gather(const uint32_t *bits, const FrontPoint *pts, int n, int s, int ns, int j,
                           int W, uint32_t *out, cudaStream_t stream);
 
+// ---- iteration counters ------------------------------------------------------
+//
+// Iterations are 1 .. I_max with I_max up to 2^32 - 1, counted in 32 bits, so a
+// counter that runs ahead of the trial wraps to 0 at the end of the longest
+// runs: a loop on t <= I_max would not end there, a schedule entry looked up
+// for iteration 0 lies 2^32 - 1 entries past the first, and a target past the
+// end would pass for an early one.
+
+// Whether iteration t (one past an iteration of the run, or 1) is in the run.
+__host__ __device__ inline bool in_run(uint32_t t, uint32_t I_max) { return t - 1u < I_max; }
+// Whether iteration t + ahead is in the run; t is.
+__host__ __device__ inline bool in_run_ahead(uint32_t t, uint32_t ahead, uint32_t I_max) {
+  return ahead <= I_max - t;
+}
+// Schedule entry of iteration q: the last one is held from iteration nsched
+// on.  (q = 0, an iteration past 2^32 - 1, gets that one too; nobody reads it.)
+__host__ __device__ inline uint32_t sched_entry(uint32_t q, uint32_t nsched) {
+  return q - 1u < nsched - 1u ? q - 1u : nsched - 1u;
+}
+// A ring of schedule entries and draws holds the iterations from .. filled, at
+// most 128 of them.  Before it is extended for t >= from (nothing before t is
+// needed again): the last iteration before those to add.
+__host__ __device__ inline uint32_t ring_skip(uint32_t filled, uint32_t from, uint32_t t) {
+  return t - from > filled + 1u - from ? t - 1u : filled;
+}
+// The ring is extended by 32 at a time while this holds, until it has t ..
+// t + 47.
+__host__ __device__ inline bool ring_short(uint32_t filled, uint32_t t) {
+  return (int32_t)(t + 48u - filled) > 0;
+}
+
 // Sets the thread-local message that moda_last_error() returns.
 void set_last_error(const char *msg);
 inline void set_last_error(const std::string &msg) { set_last_error(msg.c_str()); }

@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
   const double s_min = A.s1 < A.s2 ? A.s1 : A.s2, s_max = A.s1 < A.s2 ? A.s2 : A.s1;
   auto fill_rings = [&](uint32_t first) {
     const uint32_t it = first + (uint32_t)(lane & 7);
-    const uint32_t sn = (it <= nsched ? it : nsched) - 1;
+    const uint32_t sn = sched_entry(it, nsched);
     const double sd = A.sch_delta[sn];
     int64_t slo = A.sch_lo[sn], shi = A.sch_hi[sn];
     double lod = 0, hid = 0;
@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
     }
   }
 
-  for (uint32_t t = 1; t <= I_max; ++t) {
+  for (uint32_t t = 1; in_run(t, I_max); ++t) {
     const int buf = (int)(t & 1u);
     // this iteration's jump record: settled by warp A before the barrier,
     // read by the other warps after it
@@ -746,7 +746,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
         // the copy engine only by a later barrier.
         const uint32_t tt = t + (uint32_t)LA;
         const int b = pb_next;
-        bool issue = cEscape == 0 && acount > 0 && flip_streak < 3 && tt <= I_max;
+        bool issue = cEscape == 0 && acount > 0 && flip_streak < 3 &&
+                     in_run_ahead(t, (uint32_t)LA, I_max);
         int slot_p = 0;
         if (issue) {
           slot_p = pick(sRnd[(tt % kRing) * 4 + 1], acount);
@@ -779,7 +780,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
         }
         sPf[tt & 7] = PfRec{issue ? (int)t : 0, slot_p, (int)par, 0};
       } else if (!NARROW && fc && lane == 0 && cEscape == 0 && acount > 0 &&
-                 t + 2 <= I_max) {
+                 in_run_ahead(t, 2u, I_max)) {
         // Records read in place (no prefetch buffers; the large 16-byte
         // records of the int64 variant): bring the record and state of the
         // member a jump two iterations ahead would land on into L2.  Only a

@@ -157,7 +157,7 @@ __global__ void __maxnreg__(N == 4 ? 80 : 96) qubo_kernel(const QArgs A) {
   }
   auto fill = [&](uint32_t first) {  // iterations first .. first + 31 (one warp)
     const uint32_t q = first + (uint32_t)lane;
-    const uint32_t sn = (q <= nsched ? q : nsched) - 1u;
+    const uint32_t sn = sched_entry(q, nsched);
     QRing e;
     e.delta = A.sch_delta[sn];
     e.cln = accept_scale(e.delta);
@@ -469,9 +469,9 @@ __global__ void __maxnreg__(N == 4 ? 80 : 96) qubo_kernel(const QArgs A) {
         for (int q = lane; q < W; q += 32) gB[(size_t)target * W + q] = sX[q];
       __syncwarp();
     };
-    auto refill = [&](uint32_t t) {  // the ring holds t .. t + 47 at least
-      if (filled + 1u < t) filled = t - 1u;
-      while (filled < t + 48u) {
+    auto refill = [&](uint32_t from, uint32_t t) {  // the ring holds t .. t + 47 at least
+      filled = ring_skip(filled, from, t);
+      while (ring_short(filled, t)) {
         fill(filled + 1u);
         filled += 32u;
       }
@@ -492,7 +492,7 @@ __global__ void __maxnreg__(N == 4 ? 80 : 96) qubo_kernel(const QArgs A) {
           if (p1) store(t);
           break;
         }
-        refill(t + 2u);
+        refill(t, t + 2u);
         ++t;
         continue;
       }
@@ -502,11 +502,12 @@ __global__ void __maxnreg__(N == 4 ? 80 : 96) qubo_kernel(const QArgs A) {
       __syncthreads();
       const uint32_t mode = uni(sJ[0]);
       const int slot = uni((int)sJ[2]);
+      const uint32_t from = t;
       t = uni(sJ[1]);
       if (mode == kQEnd || mode == kQLoad)  // the member the jumps ended on (written here)
         for (int q = lane; q < W; q += 32) sX[q] = gB[(size_t)slot * W + q];
       if (mode == kQEnd || mode == kQStayEnd) break;
-      refill(t);
+      refill(from, t);
       if (mode == kQLoad) {
         if (gR != nullptr) __syncthreads();
         else rebuild(false);

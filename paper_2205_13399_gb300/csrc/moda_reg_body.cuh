@@ -214,7 +214,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   // and the select draw (0, q, replica, select).
   auto fill = [&](uint32_t first) {
     const uint32_t q = first + (uint32_t)lane;
-    const uint32_t sn = (q <= nsched ? q : nsched) - 1u;
+    const uint32_t sn = sched_entry(q, nsched);
     RRing e;
     e.delta = R.sch_delta[sn];
     e.cln = accept_scale(e.delta);
@@ -1024,9 +1024,9 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       }
       __syncwarp();
     };
-    auto refill = [&](uint32_t t) {  // the ring holds t .. t + 47 at least
-      if (filled + 1u < t) filled = t - 1u;
-      while (filled < t + 48u) {
+    auto refill = [&](uint32_t from, uint32_t t) {  // the ring holds t .. t + 47 at least
+      filled = ring_skip(filled, from, t);
+      while (ring_short(filled, t)) {
         fill(filled + 1u);
         filled += 32u;
       }
@@ -1051,7 +1051,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
           if (EXT) snapshots(t);
           break;
         }
-        refill(t + 2u);
+        refill(t, t + 2u);
         ++t;
         continue;
       }
@@ -1061,13 +1061,14 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       __syncthreads();
       const uint32_t mode = uni(sJ[0]);
       const int slot = uni((int)sJ[2]);
+      const uint32_t from = t;
       t = uni(sJ[1]);
       if (EXT) snapshots(mode == kRegEnd || mode == kRegStayEnd ? I_max : t - 1u);
       if (mode == kRegEnd || mode == kRegRebuild)  // the member the jumps ended on
         for (int q = lane; q < W; q += 32) sX[q] = gB[(size_t)slot * W + q];  // (written here)
       if (mode == kRegEnd || mode == kRegStayEnd) break;
-      if (mode == kRegRebuild) rebuild(false, [&] { refill(t); });
-      else refill(t);
+      if (mode == kRegRebuild) rebuild(false, [&] { refill(from, t); });
+      else refill(from, t);
       if (D > 0) __syncthreads();  // draws
     }
     __syncwarp();

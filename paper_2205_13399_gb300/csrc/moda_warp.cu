@@ -226,7 +226,7 @@ __device__ bool team_run(const WarpRun &R, const int row, const Team &T, const W
   // exploit purposes.
   auto fill = [&](uint32_t first) {
     const uint32_t q = first + (uint32_t)lane;
-    const uint32_t sn = (q <= nsched ? q : nsched) - 1u;
+    const uint32_t sn = sched_entry(q, nsched);
     WRing e;
     e.delta = R.sch_delta[sn];
     e.deltaf = __double2float_rn(e.delta);
@@ -455,9 +455,9 @@ __device__ bool team_run(const WarpRun &R, const int row, const Team &T, const W
   // issued_to are written (none for 1 .. LA).
   uint32_t issued_to = (uint32_t)LA;
   uint32_t t = 1, rnd = 0;
-  while (t <= I_max) {
+  while (in_run(t, I_max)) {
     if (scribe)  // entries read before this round's barrier were written in earlier rounds
-      while (filled < t + 48u) {
+      while (ring_short(filled, t)) {
         fill(filled + 1u);
         filled += 32u;
       }
@@ -515,7 +515,8 @@ __device__ bool team_run(const WarpRun &R, const int row, const Team &T, const W
       const uint32_t tt = issued_to + 1u + (uint32_t)lane;
       int sp = 0;
       bool want = false;
-      if (lane < nI && acount > 0 && flip_streak < 3 && tt <= I_max) {
+      if (lane < nI && acount > 0 && flip_streak < 3 &&
+          in_run_ahead(t, tt - t, I_max)) {
         sp = pick(ring[tt % kWarpRing].rst, acount);
         // a slot written in the previous iteration is left alone: warps
         // still writing it are ordered before the copy only by the next
