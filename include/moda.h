@@ -374,12 +374,15 @@ moda_status moda_autotune(moda_instance inst, const moda_params *params, int32_t
  * A queue of anneal requests served as they arrive (not in the paper:
  * serving many bi-objective QAP solves on one GPU).  A native thread of the
  * server admits waiting requests in arrival order while the device buffers
- * of the runs in flight (the bytes moda_anneal would allocate for each) fit
- * `hbm_budget`, and launches each admitted request at once on a stream of
+ * of the runs in flight fit `hbm_budget` (the bytes moda_anneal would
+ * allocate for each; for runs of the register annealer that jump to their
+ * archives, unless field_cache = 2, also the scratch that moda_read_archive
+ * takes for the whole front), and launches each admitted request at once on a stream of
  * its own (or on `cuda_stream` if not NULL, which orders them), so new
  * requests join the ones already running instead of waiting for a batch.
- * A request whose buffers with the field cache do not fit runs without it
- * (identical results) once nothing else is running, if that fits; it fails
+ * A request whose buffers with the field cache (or that scratch) do not fit
+ * runs without it (identical results) once nothing else is running, if that
+ * fits; it fails
  * with MODA_ENOMEM when it cannot fit even then.  A request whose device
  * allocation fails while other runs hold memory waits for them.  Each request's results equal those of moda_anneal on
  * the same instance and params.

@@ -363,6 +363,23 @@ bool prescribes_team(const moda_params *p) {
   return p->prefetch > 0 || p->block_threads > 0 || p->field_cache == 1 || p->cache_slots > 0;
 }
 
+// The kernel that runs a request (and, for the register annealer, how it fits).
+// The options that the block engine would refuse are left to it to refuse.
+enum class Kernel { kBlock, kTeam, kRegister };
+Kernel kernel_of(moda_instance inst, const moda_params *p, moda::RegFit *fit) {
+  *fit = moda::RegFit{};
+  const bool narrow = moda::narrow_ok(inst->n, inst->b1, inst->b2, inst->w1, inst->w2);
+  if (uses_warp(p)) {
+    if (!prescribes_team(p)) *fit = reg_plan(inst, p, narrow);
+    return fit->se > 0 ? Kernel::kRegister : Kernel::kTeam;
+  }
+  if (reg_extension(p) && p->field_cache >= 0 && p->field_cache <= 2 &&
+      (p->normalize == 0 || p->normalize == 1) && p->snapshot_every >= 0 &&
+      (p->snapshot_every == 0 || p->I_max / p->snapshot_every <= 1000000))
+    *fit = reg_plan(inst, p, narrow);
+  return fit->se > 0 ? Kernel::kRegister : Kernel::kBlock;
+}
+
 }  // namespace
 
 extern "C" {
@@ -542,11 +559,11 @@ moda_status moda_instance_info(moda_instance inst, int32_t *n, int64_t *w1,
 
 namespace {
 
-// The warp annealer's part of prepare_run: validated params, the run's
+// The warp and register annealers' part of prepare_run: validated params, the run's
 // buffers, and its WarpRun descriptor (field-cache slots, on-chip archive
 // energies and the work list are settled when the launch is planned).
-moda_status prepare_warp_run(moda_instance inst, const moda_params *p, cudaStream_t stream,
-                             moda_run *out, Prepared *pl) {
+moda_status prepare_warp_run(moda_instance inst, const moda_params *p, const moda::RegFit &fit,
+                             cudaStream_t stream, moda_run *out, Prepared *pl) {
   const int m = inst->m;
   if (p->field_cache < 0 || p->field_cache > 2)
     return fail(MODA_EINVAL, "field_cache must be 0 (auto), 1 (on) or 2 (off)");
@@ -565,8 +582,6 @@ moda_status prepare_warp_run(moda_instance inst, const moda_params *p, cudaStrea
   r->stream = stream;
   r->warp = true;
   const bool narrow = moda::narrow_ok(inst->n, inst->b1, inst->b2, inst->w1, inst->w2);
-  moda::RegFit fit;
-  if (!prescribes_team(p)) fit = reg_plan(inst, p, narrow);
   r->reg = fit.se > 0;
   const size_t R = r->R, s = r->s, W = inst->W;
   moda_status st = MODA_OK;
@@ -703,13 +718,9 @@ moda_status prepare_run(moda_instance inst, const moda_params *p,
     return fail(MODA_EUNSUPPORTED,
                 "the warp engine needs the archive escape without normalize, "
                 "snapshot_every or fast_forward");
-  if (uses_warp(p)) return prepare_warp_run(inst, p, stream, out, pl);
-  // (checked here as the block engine checks them below)
-  if (reg_extension(p) && p->field_cache >= 0 && p->field_cache <= 2 &&
-      (p->normalize == 0 || p->normalize == 1) && p->snapshot_every >= 0 &&
-      (p->snapshot_every == 0 || p->I_max / p->snapshot_every <= 1000000) &&
-      reg_plan(inst, p, moda::narrow_ok(inst->n, inst->b1, inst->b2, inst->w1, inst->w2)).se > 0)
-    return prepare_warp_run(inst, p, stream, out, pl);
+  moda::RegFit fit;
+  if (kernel_of(inst, p, &fit) != Kernel::kBlock)
+    return prepare_warp_run(inst, p, fit, stream, out, pl);
 
   // Block shape: B rounds of T threads own the bits, B * T >= m.
   static const int kRounds[] = {1, 2, 3, 4, 6, 8};
@@ -923,21 +934,28 @@ moda_status prepare_run(moda_instance inst, const moda_params *p,
   return MODA_OK;
 }
 
-// Device bytes a run of `p` on `inst` allocates, with or without the field
-// cache (the same buffers as prepare_run).
+// Device bytes a run of `p` on `inst` allocates (the same buffers as
+// prepare_run), and with `cache` those that it can do without: the field cache
+// of the kernels that have one.  The register annealer has none; what counts
+// for its runs, under the same options, is the scratch that archive_front
+// takes while the whole front is read (two lists of points and their states).
 size_t run_bytes(moda_instance inst, const moda_params &p, bool cache) {
   const size_t R = (size_t)p.replicas, m = (size_t)inst->m, W = (size_t)inst->W;
   const size_t s = p.archive_size > 0 ? (size_t)p.archive_size : m;
+  moda::RegFit fit;
+  const Kernel kernel = kernel_of(inst, &p, &fit);
   const bool narrow = moda::narrow_ok(inst->n, inst->b1, inst->b2, inst->w1, inst->w2);
   size_t b = R * s * 2 * sizeof(int64_t) + R * s * W * sizeof(uint32_t) + 32 +
              R * sizeof(int32_t) + R * W * sizeof(uint32_t) + R * 2 * sizeof(int64_t) +
              R * moda::kStats * sizeof(int64_t) + sizeof(int32_t);
-  if (cache && uses_warp(&p)) {
-    // the field caches of up to R resident teams
+  if (kernel == Kernel::kRegister && s > (size_t)fit.se) b += R * s * sizeof(uint32_t);
+  const bool jumps = p.escape == MODA_ESC_ARCHIVE && p.field_cache != 2;
+  if (cache && kernel == Kernel::kTeam)  // the field caches of up to R resident teams
     b += R * moda::align_up(moda::warp_cache_bytes(inst->n, (int)m, warp_slots(inst, p)), 256);
-  } else if (cache && p.escape == MODA_ESC_ARCHIVE && p.field_cache != 2) {
+  else if (cache && kernel == Kernel::kRegister && jumps)
+    b += R * s * (2 * sizeof(moda::FrontPoint) + W * sizeof(uint32_t)) + 32;
+  else if (cache && kernel == Kernel::kBlock && jumps)
     b += R * s * moda::slot_layout((int)m, narrow).bytes;
-  }
   if (p.trace && p.I_max > 0) b += R * (size_t)p.I_max * 3 * sizeof(int64_t);
   if (p.snapshot_every > 0) {
     const size_t ns = (size_t)(p.I_max / p.snapshot_every);
@@ -1610,8 +1628,10 @@ moda_status moda_anneal_batch(const moda_instance *insts, const moda_params *par
                                    " bytes of run buffers; " + std::to_string(free_b) + " free");
     size_t budget = free_b / 10 * 6 > lean ? free_b / 10 * 6 - lean : 0;
     std::vector<std::pair<size_t, int32_t>> want;
+    moda::RegFit fit;
     for (int32_t i = 0; i < count; ++i)
-      if (!uses_warp(&prm[i]) && prm[i].field_cache == 0 && prm[i].escape == MODA_ESC_ARCHIVE)
+      if (prm[i].field_cache == 0 && prm[i].escape == MODA_ESC_ARCHIVE &&
+          kernel_of(insts[i], &prm[i], &fit) == Kernel::kBlock)
         want.emplace_back(run_bytes(insts[i], prm[i], true) - run_bytes(insts[i], prm[i], false),
                           i);
     std::sort(want.begin(), want.end());
@@ -1662,13 +1682,16 @@ moda_status moda_anneal_batch(const moda_instance *insts, const moda_params *par
     classes[std::make_tuple(pls[i].narrow ? 1 : 0, 0, -cls, runs[i]->prm.prefetch)].push_back(i);
   }
   std::vector<WarpGroup> groups;
+  size_t teams = 0;  // launches of the team annealer, which share the budget of the caches
   for (auto &kv : classes) {
     WarpGroup G;
     G.idx = kv.second;
+    if (!runs[G.idx[0]]->reg) ++teams;
     groups.push_back(std::move(G));
   }
   for (WarpGroup &G : groups) {
-    moda_status st = plan_warp_group(runs, pls, G, stream, warp_budget / groups.size());
+    moda_status st =
+        plan_warp_group(runs, pls, G, stream, warp_budget / std::max<size_t>(teams, 1));
     if (st != MODA_OK) {
       const std::string msg = g_error;
       cudaStreamSynchronize(stream);
@@ -1911,6 +1934,8 @@ void server_loop(moda_server_s *S) {
         q->msg = g_error;
         continue;
       }
+      // (a register run's front scratch, counted while the run is held)
+      if (r->reg) r->bytes += run_bytes(q->inst, prm, true) - run_bytes(q->inst, prm, false);
       q->run = r;
       q->bytes = r->bytes;
       q->state = Request::kRunning;
