@@ -403,8 +403,8 @@ moda_status moda_server_submit(moda_server srv, moda_instance inst,
 moda_status moda_server_poll(moda_server srv, int64_t ticket, moda_run *done);
 /* Queue state: requests waiting, requests running (launched and not yet seen
  * finished: a poll sees its own request's finish, and the server looks at all
- * of them while a request waits for memory), bytes of their buffers and the
- * budget (any pointer may be NULL). */
+ * of them every 50 ms, every 100 us while a request waits for memory), bytes
+ * of their buffers and the budget (any pointer may be NULL). */
 moda_status moda_server_info(moda_server srv, int64_t *pending, int64_t *running,
                              size_t *bytes_in_use, size_t *budget);
 void moda_server_destroy(moda_server srv);

@@ -1827,6 +1827,7 @@ struct moda_server_s {
 namespace {
 
 constexpr int kServerStreams = 32;
+constexpr std::chrono::milliseconds kServerLook(50);
 
 // Looks whether running request i has finished (caller holds the lock): if
 // so it leaves the list of running ones.
@@ -1848,19 +1849,26 @@ bool server_retire(moda_server_s *S, size_t i) {
 
 // The server's thread: admits waiting requests in arrival order while their
 // buffers fit the budget, each on a stream of its own, so a request starts
-// as soon as memory allows, beside those already running.  It sleeps until a
-// request arrives: a run's finish is noticed by its poll (moda_server_poll
-// looks at the run's event itself), and here only while a request waits for
-// memory or the server stops.  (Looking every 100 us instead woke the thread
-// 10,000 times a second under the lock that submit and poll take.)
+// as soon as memory allows, beside those already running.  A run's finish is
+// noticed by its poll (moda_server_poll looks at the run's event itself); the
+// thread looks at all of them every 100 us while a request waits for memory or
+// the server stops, else every kServerLook, so that the count of running
+// requests falls for a program that only watches it.  (Looking every 100 us
+// always woke the thread 10,000 times a second under the lock that submit and
+// poll take.)
 void server_loop(moda_server_s *S) {
   cudaSetDevice(S->device);
   std::unique_lock<std::mutex> lock(S->mu);
   bool blocked = false;  // the first waiting request did not fit
+  auto looked = std::chrono::steady_clock::now();
   for (;;) {
-    if (blocked || S->stopping)
+    const auto now = std::chrono::steady_clock::now();
+    if (S->running.empty()) looked = now;
+    if (blocked || S->stopping || now - looked >= kServerLook) {
       for (size_t i = 0; i < S->running.size();)
         if (!server_retire(S, i)) ++i;
+      looked = now;
+    }
     blocked = false;
     while (!S->pending.empty()) {
       std::shared_ptr<Request> q = S->pending.front();
@@ -1945,10 +1953,13 @@ void server_loop(moda_server_s *S) {
       S->running.push_back(q);
     }
     if (S->stopping && S->pending.empty() && S->running.empty()) break;
+    auto wake = [&] { return S->stopping || !S->pending.empty(); };
     if (blocked || S->stopping)
       S->cv.wait_for(lock, std::chrono::microseconds(100));
+    else if (!S->running.empty())
+      S->cv.wait_until(lock, looked + kServerLook, wake);
     else
-      S->cv.wait(lock, [&] { return S->stopping || !S->pending.empty(); });
+      S->cv.wait(lock, wake);
   }
 }
 

@@ -68,3 +68,16 @@ def test_the_budget_covers_every_buffer():
         assert time.time() - t0 < 60
     assert most <= 2 * one - 1
     srv.close()
+
+
+def test_running_falls_without_a_poll():
+    """A program that watches the server's counters until it is idle."""
+    from paper_2205_13399_gb300 import moda
+    qi = inputs.uniform_instance(8, index=1, workload="P8")
+    inst = moda.Instance(qi.F1, qi.F2, qi.D)
+    srv = moda.Server()
+    t = srv.submit(inst, replicas=2, I_max=2000, seed=1)
+    _until(lambda: srv.info()["pending"] == 0)
+    _until(lambda: srv.info()["running"] == 0, seconds=5.0)
+    assert srv.poll(t) is not None
+    srv.close()
