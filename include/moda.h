@@ -361,11 +361,12 @@ void moda_qrun_destroy(moda_qrun run);
  * deltaf, on at most one replica per SM); for the warp engine, prefetch
  * distances 0, 2, 6, 10 and 14 of the team annealer on the request's own
  * replicas and, where the engine is left open and no layout is prescribed,
- * the register annealer (prefetch 0).  Writes into *best a copy of *params
- * with the fastest block_threads and prefetch; *best_ms (if not NULL)
- * receives the winning trial's time.  Results of a run do not depend on these two
- * fields, so tuning never changes what an anneal computes.  Blocks the
- * calling thread while the trials run on cuda_stream. */
+ * the register annealer (prefetch 0), which is also a candidate beside the
+ * block shapes for the options it takes from the block engine.  Writes into
+ * *best a copy of *params with the fastest block_threads and prefetch; *best_ms
+ * (if not NULL) receives the winning trial's time.  Results of a run do not
+ * depend on these two fields, so tuning never changes what an anneal computes.
+ * Blocks the calling thread while the trials run on cuda_stream. */
 moda_status moda_autotune(moda_instance inst, const moda_params *params, int32_t trial_iters,
                           void *cuda_stream, moda_params *best, float *best_ms);
 

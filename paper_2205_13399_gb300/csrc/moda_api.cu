@@ -2280,22 +2280,32 @@ moda_status moda_autotune(moda_instance inst, const moda_params *params, int32_t
   bool found = false;
   float fastest = 0.f;
   moda_params winner = *params;
-  for (int32_t T : shapes)
-    for (int32_t pf : prefetches) {
-      trial.block_threads = T;
-      trial.prefetch = pf;
-      moda_run r = nullptr;
-      if (moda_anneal(inst, &trial, stream, &r) != MODA_OK) continue;  // does not fit
-      float ms = 0.f;
-      const bool ok = moda_wait(r, -1) == MODA_OK && moda_run_elapsed_ms(r, &ms) == MODA_OK;
-      moda_destroy_run(r);
-      if (ok && (!found || ms < fastest)) {
-        found = true;
-        fastest = ms;
-        winner.block_threads = T;
-        winner.prefetch = pf;
-      }
+  auto time_trial = [&](int32_t T, int32_t pf) {
+    trial.block_threads = T;
+    trial.prefetch = pf;
+    moda_run r = nullptr;
+    if (moda_anneal(inst, &trial, stream, &r) != MODA_OK) return;  // does not fit
+    float ms = 0.f;
+    const bool ok = moda_wait(r, -1) == MODA_OK && moda_run_elapsed_ms(r, &ms) == MODA_OK;
+    moda_destroy_run(r);
+    if (ok && (!found || ms < fastest)) {
+      found = true;
+      fastest = ms;
+      winner.block_threads = T;
+      winner.prefetch = pf;
     }
+  };
+  // A request that the register annealer takes while no shape is prescribed is
+  // a candidate as it stands (with its snapshots: without them a request of
+  // that option alone would run on another kernel).
+  moda::RegFit fit;
+  if (kernel_of(inst, params, &fit) == Kernel::kRegister) {
+    trial.snapshot_every = params->snapshot_every;
+    time_trial(0, 0);
+    trial.snapshot_every = 0;
+  }
+  for (int32_t T : shapes)
+    for (int32_t pf : prefetches) time_trial(T, pf);
   if (!found) return fail(MODA_EUNSUPPORTED, "no candidate shape runs this instance");
   *best = winner;
   if (best_ms) *best_ms = fastest;
