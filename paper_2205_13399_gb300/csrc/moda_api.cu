@@ -1444,6 +1444,24 @@ moda_status moda_read_trace(moda_run r, int32_t rep, int64_t *trace) {
 
 namespace {
 
+// Device scratch of a read, given back in stream order.
+struct ReadBuffer {
+  cudaStream_t st;
+  void *p = nullptr;
+  ~ReadBuffer() {
+    if (p) cudaFreeAsync(p, st);
+  }
+  // false: no memory for it (the read then goes through the host)
+  cudaError_t get(size_t bytes, bool *have) {
+    const cudaError_t e = cudaMallocAsync(&p, bytes, st);
+    *have = e == cudaSuccess;
+    if (e != cudaErrorMemoryAllocation) return e;
+    p = nullptr;
+    cudaGetLastError();  // not an error of the calls that follow
+    return cudaSuccess;
+  }
+};
+
 // The non-dominated members of replica `rep` (or all, rep == -1) of an
 // archive held on the device as counts[q * ns + j], energies at
 // E + (q * ns + j) * s * 2 and states at bits + (q * ns + j) * s * W: the
@@ -1463,17 +1481,12 @@ moda_status archive_front(moda_run r, int32_t rep, moda_point *pts, int32_t cap,
   MODA_CUDA(cudaStreamSynchronize(st));
   size_t most = 0;
   for (int32_t q : cnt) most += (size_t)std::min(std::max(q, 0), s);
-  struct Buffer {  // device scratch, given back in stream order
-    cudaStream_t st;
-    void *p = nullptr;
-    ~Buffer() {
-      if (p) cudaFreeAsync(p, st);
-    }
-  } list{st}, words{st};
+  ReadBuffer list{st}, words{st};
   std::vector<moda::FrontPoint> c;
-  if (most > 0) {
-    const size_t head = 16;
-    MODA_CUDA(cudaMallocAsync(&list.p, head + most * sizeof(moda::FrontPoint), st));
+  const size_t head = 16;
+  bool have = false;
+  if (most > 0) MODA_CUDA(list.get(head + most * sizeof(moda::FrontPoint), &have));
+  if (have) {  // each replica's own front
     auto *total = static_cast<uint32_t *>(list.p);
     auto *out = reinterpret_cast<moda::FrontPoint *>(static_cast<unsigned char *>(list.p) + head);
     MODA_CUDA(cudaMemsetAsync(total, 0, sizeof(uint32_t), st));
@@ -1485,6 +1498,17 @@ moda_status archive_front(moda_run r, int32_t rep, moda_point *pts, int32_t cap,
     MODA_CUDA(cudaMemcpyAsync(c.data(), out, sizeof(moda::FrontPoint) * got,
                               cudaMemcpyDeviceToHost, st));
     MODA_CUDA(cudaStreamSynchronize(st));
+  } else if (most > 0) {  // every member
+    std::vector<int64_t> E;
+    for (int q = first; q < last; ++q) {
+      const int k = std::min(std::max(cnt[q - first], 0), s);
+      if (k == 0) continue;
+      E.resize(2 * (size_t)k);
+      MODA_CUDA(cudaMemcpyAsync(E.data(), dE + ((size_t)q * ns + j) * s * 2,
+                                sizeof(int64_t) * E.size(), cudaMemcpyDeviceToHost, st));
+      MODA_CUDA(cudaStreamSynchronize(st));
+      for (int y = 0; y < k; ++y) c.push_back({E[2 * y], E[2 * y + 1], q, y});
+    }
   }
   std::sort(c.begin(), c.end(), [](const moda::FrontPoint &a, const moda::FrontPoint &b) {
     if (a.e1 != b.e1) return a.e1 < b.e1;
@@ -1507,11 +1531,12 @@ moda_status archive_front(moda_run r, int32_t rep, moda_point *pts, int32_t cap,
   }
   *count = (int32_t)keep.size();
   const int wr = std::min<int32_t>(cap, (int32_t)keep.size());
-  // their states, in one copy
+  // their states, in one copy (or one each)
   std::vector<uint32_t> state((size_t)wr * W);
-  if (wr > 0) {
-    const size_t pb = moda::align_up(sizeof(moda::FrontPoint) * (size_t)wr, 16);
-    MODA_CUDA(cudaMallocAsync(&words.p, pb + sizeof(uint32_t) * state.size(), st));
+  const size_t pb = moda::align_up(sizeof(moda::FrontPoint) * (size_t)wr, 16);
+  have = false;
+  if (wr > 0) MODA_CUDA(words.get(pb + sizeof(uint32_t) * state.size(), &have));
+  if (have) {
     auto *pts_d = static_cast<moda::FrontPoint *>(words.p);
     auto *out = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(words.p) + pb);
     MODA_CUDA(cudaMemcpyAsync(pts_d, keep.data(), sizeof(moda::FrontPoint) * (size_t)wr,
@@ -1519,8 +1544,14 @@ moda_status archive_front(moda_run r, int32_t rep, moda_point *pts, int32_t cap,
     MODA_CUDA(moda::launch_gather(dbits, pts_d, wr, s, (int)ns, (int)j, W, out, st));
     MODA_CUDA(cudaMemcpyAsync(state.data(), out, sizeof(uint32_t) * state.size(),
                               cudaMemcpyDeviceToHost, st));
-    MODA_CUDA(cudaStreamSynchronize(st));
+  } else {
+    for (int k = 0; k < wr; ++k)
+      MODA_CUDA(cudaMemcpyAsync(
+          state.data() + (size_t)k * W,
+          dbits + (((size_t)keep[k].rep * ns + j) * s + keep[k].slot) * W,
+          sizeof(uint32_t) * W, cudaMemcpyDeviceToHost, st));
   }
+  if (wr > 0) MODA_CUDA(cudaStreamSynchronize(st));
   for (int k = 0; k < wr; ++k) {
     const moda::FrontPoint &q = keep[k];
     const uint32_t *word = state.data() + (size_t)k * W;
