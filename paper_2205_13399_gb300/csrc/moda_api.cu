@@ -226,24 +226,41 @@ namespace {
 // retiring one run never stalls the others.  The default pool of each
 // device keeps freed memory for reuse.
 std::mutex g_pool_mutex;
-std::map<int, cudaStream_t> g_free_streams;
+struct LibStreams {
+  cudaStream_t free = nullptr, copy = nullptr;
+};
+std::map<int, LibStreams> g_lib_streams;
 
-// Per device: a library stream for frees of finished runs, and the pool
-// set to keep its memory.
-cudaStream_t free_stream(int dev) {
+// Per device: a library stream for frees of finished runs and the kernels
+// that read their fronts, one for instance uploads and plain copies (which
+// never wait for a kernel), and the pool set to keep its memory.  The first
+// has the highest priority: the blocks of a front then go ahead of those that
+// other runs have not started yet.
+LibStreams lib_streams(int dev) {
   std::lock_guard<std::mutex> lock(g_pool_mutex);
-  auto it = g_free_streams.find(dev);
-  if (it != g_free_streams.end()) return it->second;
-  cudaStream_t st = nullptr;
-  if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) st = nullptr;
+  auto it = g_lib_streams.find(dev);
+  if (it != g_lib_streams.end()) return it->second;
+  LibStreams st;
+  int lo = 0, hi = 0;
+  cudaDeviceGetStreamPriorityRange(&lo, &hi);
+  if (cudaStreamCreateWithPriority(&st.free, cudaStreamNonBlocking, hi) != cudaSuccess)
+    st.free = nullptr;
+  if (cudaStreamCreateWithFlags(&st.copy, cudaStreamNonBlocking) != cudaSuccess)
+    st.copy = nullptr;
   cudaMemPool_t pool;
   if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
     uint64_t keep = UINT64_MAX;
     cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    // an allocation takes new memory rather than wait for a free that is
+    // queued behind a front
+    int no = 0;
+    cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &no);
   }
-  g_free_streams[dev] = st;
+  g_lib_streams[dev] = st;
   return st;
 }
+cudaStream_t free_stream(int dev) { return lib_streams(dev).free; }
+cudaStream_t copy_stream(int dev) { return lib_streams(dev).copy; }
 
 // Free device memory including what the pool holds unused.
 cudaError_t free_memory(int dev, size_t *free_b) {
@@ -479,7 +496,7 @@ moda_status finish_instance(moda_instance inst, const moda_penalty *pen, moda_in
   // uploads on it too: neither waits for work in flight elsewhere on the
   // device (a server creates an instance per request while others run).
   const size_t bytes = sizeof(int32_t) * nn;
-  cudaStream_t fs = free_stream(inst->device);
+  cudaStream_t fs = copy_stream(inst->device);
   void *base = nullptr;
   cudaError_t e = cudaMallocAsync(&base, 3 * bytes, fs);
   if (e == cudaSuccess) {
@@ -1444,15 +1461,15 @@ moda_status moda_read_trace(moda_run r, int32_t rep, int64_t *trace) {
 
 namespace {
 
-// Device scratch of a read, given back in stream order.
+// Device scratch of a read, given back in the order of the read's kernels.
 struct ReadBuffer {
-  cudaStream_t st;
+  cudaStream_t kernels;
   void *p = nullptr;
   ~ReadBuffer() {
-    if (p) cudaFreeAsync(p, st);
+    if (p) cudaFreeAsync(p, kernels);
   }
-  // false: no memory for it (the read then goes through the host)
-  cudaError_t get(size_t bytes, bool *have) {
+  // *have = false: no memory for it (the read then goes through the host)
+  cudaError_t get(size_t bytes, cudaStream_t st, bool *have) {
     const cudaError_t e = cudaMallocAsync(&p, bytes, st);
     *have = e == cudaSuccess;
     if (e != cudaErrorMemoryAllocation) return e;
@@ -1461,6 +1478,31 @@ struct ReadBuffer {
     return cudaSuccess;
   }
 };
+
+// Waits for what was enqueued on `st`, but not long: the kernels of a read
+// wait for room on a device that runs are filling (up to the time one of their
+// blocks takes, 100 ms and more; front and gather take 20 us alone), and
+// reading through the host takes a few milliseconds.  False: not done.
+cudaError_t read_wait(cudaStream_t st, bool *done) {
+  constexpr std::chrono::microseconds kReadWait(1000);
+  *done = false;
+  cudaEvent_t ev = nullptr;
+  cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+  if (e != cudaSuccess) return e;
+  e = cudaEventRecord(ev, st);
+  const auto t0 = std::chrono::steady_clock::now();
+  while (e == cudaSuccess) {
+    e = cudaEventQuery(ev);
+    if (e == cudaSuccess) {
+      *done = true;
+      break;
+    }
+    if (e == cudaErrorNotReady)
+      e = std::chrono::steady_clock::now() - t0 < kReadWait ? cudaSuccess : cudaErrorNotReady;
+  }
+  cudaEventDestroy(ev);
+  return e == cudaErrorNotReady ? cudaSuccess : e;
+}
 
 // The non-dominated members of replica `rep` (or all, rep == -1) of an
 // archive held on the device as counts[q * ns + j], energies at
@@ -1473,41 +1515,56 @@ moda_status archive_front(moda_run r, int32_t rep, moda_point *pts, int32_t cap,
   const int s = r->s;
   const int first = rep < 0 ? 0 : rep, last = rep < 0 ? r->R : rep + 1;
   // the archive sizes bound the packed list
-  cudaStream_t st = free_stream(r->inst->device);
+  cudaStream_t st = free_stream(r->inst->device), copies = copy_stream(r->inst->device);
   std::vector<int32_t> cnt((size_t)(last - first));
   MODA_CUDA(cudaMemcpy2DAsync(cnt.data(), sizeof(int32_t), dcnt + (size_t)first * ns + j,
                               sizeof(int32_t) * ns, sizeof(int32_t), cnt.size(),
-                              cudaMemcpyDeviceToHost, st));
-  MODA_CUDA(cudaStreamSynchronize(st));
+                              cudaMemcpyDeviceToHost, copies));
+  MODA_CUDA(cudaStreamSynchronize(copies));
   size_t most = 0;
   for (int32_t q : cnt) most += (size_t)std::min(std::max(q, 0), s);
   ReadBuffer list{st}, words{st};
   std::vector<moda::FrontPoint> c;
-  const size_t head = 16;
+  auto fetch = [&](void *to, const void *from, size_t bytes) -> cudaError_t {
+    const cudaError_t e = cudaMemcpyAsync(to, from, bytes, cudaMemcpyDeviceToHost, copies);
+    return e == cudaSuccess ? cudaStreamSynchronize(copies) : e;
+  };
   bool have = false;
-  if (most > 0) MODA_CUDA(list.get(head + most * sizeof(moda::FrontPoint), &have));
-  if (have) {  // each replica's own front
+  const size_t head = 16;
+  if (most > 0) MODA_CUDA(list.get(head + most * sizeof(moda::FrontPoint), st, &have));
+  if (have) {  // each replica's own front, behind a counter
     auto *total = static_cast<uint32_t *>(list.p);
     auto *out = reinterpret_cast<moda::FrontPoint *>(static_cast<unsigned char *>(list.p) + head);
     MODA_CUDA(cudaMemsetAsync(total, 0, sizeof(uint32_t), st));
-    MODA_CUDA(moda::launch_front(dcnt, dE, s, (int)ns, (int)j, first, last - first, out, total, st));
+    MODA_CUDA(
+        moda::launch_front(dcnt, dE, s, (int)ns, (int)j, first, last - first, out, total, st));
+    MODA_CUDA(read_wait(st, &have));
+  }
+  if (have) {
+    const auto *out = static_cast<const unsigned char *>(list.p);
     uint32_t got = 0;
-    MODA_CUDA(cudaMemcpyAsync(&got, total, sizeof(got), cudaMemcpyDeviceToHost, st));
-    MODA_CUDA(cudaStreamSynchronize(st));
+    MODA_CUDA(fetch(&got, out, sizeof(got)));
     c.resize(got);
-    MODA_CUDA(cudaMemcpyAsync(c.data(), out, sizeof(moda::FrontPoint) * got,
-                              cudaMemcpyDeviceToHost, st));
-    MODA_CUDA(cudaStreamSynchronize(st));
-  } else if (most > 0) {  // every member
-    std::vector<int64_t> E;
-    for (int q = first; q < last; ++q) {
-      const int k = std::min(std::max(cnt[q - first], 0), s);
-      if (k == 0) continue;
-      E.resize(2 * (size_t)k);
-      MODA_CUDA(cudaMemcpyAsync(E.data(), dE + ((size_t)q * ns + j) * s * 2,
-                                sizeof(int64_t) * E.size(), cudaMemcpyDeviceToHost, st));
-      MODA_CUDA(cudaStreamSynchronize(st));
-      for (int y = 0; y < k; ++y) c.push_back({E[2 * y], E[2 * y + 1], q, y});
+    MODA_CUDA(fetch(c.data(), out + head, sizeof(moda::FrontPoint) * got));
+  }
+  const bool by_host = most > 0 && !have;
+  if (by_host) {  // every member, the archives of some replicas at a time
+    const size_t longest = (size_t)std::min(*std::max_element(cnt.begin(), cnt.end()), s);
+    const size_t row = 2 * sizeof(int64_t) * longest, pitch = 2 * sizeof(int64_t) * ns * s;
+    const int rows =  // 16 MiB; one where the copy's pitch would pass its limit
+        pitch < (size_t(1) << 31) ? (int)std::max<size_t>((size_t(1) << 24) / row, 1) : 1;
+    std::vector<int64_t> E(2 * longest * (size_t)std::min(rows, last - first));
+    for (int q0 = first; q0 < last; q0 += rows) {
+      const int q1 = std::min(q0 + rows, last);
+      MODA_CUDA(cudaMemcpy2DAsync(E.data(), row, dE + ((size_t)q0 * ns + j) * s * 2,
+                                  q1 - q0 > 1 ? pitch : row, row, (size_t)(q1 - q0),
+                                  cudaMemcpyDeviceToHost, copies));
+      MODA_CUDA(cudaStreamSynchronize(copies));
+      for (int q = q0; q < q1; ++q) {
+        const int64_t *e = E.data() + 2 * longest * (size_t)(q - q0);
+        for (int y = 0; y < std::min(cnt[q - first], s); ++y)
+          c.push_back({e[2 * y], e[2 * y + 1], q, y});
+      }
     }
   }
   std::sort(c.begin(), c.end(), [](const moda::FrontPoint &a, const moda::FrontPoint &b) {
@@ -1533,25 +1590,23 @@ moda_status archive_front(moda_run r, int32_t rep, moda_point *pts, int32_t cap,
   const int wr = std::min<int32_t>(cap, (int32_t)keep.size());
   // their states, in one copy (or one each)
   std::vector<uint32_t> state((size_t)wr * W);
-  const size_t pb = moda::align_up(sizeof(moda::FrontPoint) * (size_t)wr, 16);
+  const size_t list_bytes = sizeof(moda::FrontPoint) * (size_t)wr;
+  const size_t pb = moda::align_up(list_bytes, 16), state_bytes = sizeof(uint32_t) * state.size();
   have = false;
-  if (wr > 0) MODA_CUDA(words.get(pb + sizeof(uint32_t) * state.size(), &have));
+  if (wr > 0 && !by_host) MODA_CUDA(words.get(pb + state_bytes, copies, &have));
   if (have) {
-    auto *pts_d = static_cast<moda::FrontPoint *>(words.p);
     auto *out = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(words.p) + pb);
-    MODA_CUDA(cudaMemcpyAsync(pts_d, keep.data(), sizeof(moda::FrontPoint) * (size_t)wr,
-                              cudaMemcpyHostToDevice, st));
-    MODA_CUDA(moda::launch_gather(dbits, pts_d, wr, s, (int)ns, (int)j, W, out, st));
-    MODA_CUDA(cudaMemcpyAsync(state.data(), out, sizeof(uint32_t) * state.size(),
-                              cudaMemcpyDeviceToHost, st));
-  } else {
-    for (int k = 0; k < wr; ++k)
-      MODA_CUDA(cudaMemcpyAsync(
-          state.data() + (size_t)k * W,
-          dbits + (((size_t)keep[k].rep * ns + j) * s + keep[k].slot) * W,
-          sizeof(uint32_t) * W, cudaMemcpyDeviceToHost, st));
+    MODA_CUDA(cudaMemcpyAsync(words.p, keep.data(), list_bytes, cudaMemcpyHostToDevice, copies));
+    MODA_CUDA(cudaStreamSynchronize(copies));  // (the kernel runs on another stream)
+    MODA_CUDA(moda::launch_gather(dbits, static_cast<moda::FrontPoint *>(words.p), wr, s, (int)ns,
+                                  (int)j, W, out, st));
+    MODA_CUDA(read_wait(st, &have));
+    if (have) MODA_CUDA(fetch(state.data(), out, state_bytes));
   }
-  if (wr > 0) MODA_CUDA(cudaStreamSynchronize(st));
+  for (int k = 0; !have && k < wr; ++k)
+    MODA_CUDA(fetch(state.data() + (size_t)k * W,
+                    dbits + (((size_t)keep[k].rep * ns + j) * s + keep[k].slot) * W,
+                    sizeof(uint32_t) * W));
   for (int k = 0; k < wr; ++k) {
     const moda::FrontPoint &q = keep[k];
     const uint32_t *word = state.data() + (size_t)k * W;

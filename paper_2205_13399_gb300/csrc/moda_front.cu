@@ -15,7 +15,10 @@
 namespace moda {
 namespace {
 
-constexpr int kFrontTile = 256;
+// Threads of a block: few enough to fit beside the annealing blocks (n = 75, one
+// an SM: a read beside such a run took 89 ms with 256, 0.5 with 128; alone 0.47
+// and 0.56).
+constexpr int kFrontTile = 128;
 
 __global__ void __launch_bounds__(kFrontTile) front_kernel(const int32_t *counts, const int64_t *E,
                                                            int s, int ns, int j, int first,
