@@ -44,6 +44,7 @@ namespace {
 constexpr int kMaxK = 3;
 constexpr int kMaxQBits = 4096;
 constexpr int kQRing = 128;
+constexpr int kQPad = 256;  // entries after the matrices: workers read whole words past the last row
 constexpr int kQSpare = 4;  // records beyond one per slot: flips in flight
 
 enum : uint32_t { kQEnd = 0, kQLoad = 1, kQStay = 2, kQStayEnd = 3 };
@@ -94,7 +95,7 @@ struct QArgs {
   int64_t I_max, beta;
   uint32_t replica_base, seed_lo, seed_hi;
   int32_t accept, archive, escape;
-  const int32_t *P;          // [K][m][m]: P_j = Q_j + Q_j^T, diagonal Q_pp
+  const int32_t *P;          // [K][m][m]: P_j = Q_j + Q_j^T, diagonal Q_pp; kQPad more
   const double *sch_delta;
   const int64_t *sch_lo, *sch_hi;
   const double *table;
@@ -181,42 +182,64 @@ __global__ void __maxnreg__(N == 4 ? 80 : 96) qubo_kernel(const QArgs A) {
   uint32_t xn = 0u;  // bit k: the lane's bit of word k
   const int w0 = wid < G ? wid * N : W;
   auto bit_of = [&](int k) { return 32 * (w0 + k) + lane; };
-  // Delta E of the state in sX from scratch: Delta E_j(q) = (1 - 2 x_q)
-  // (P_j[q][q] + sum_{r in x, r != q} P_j[r][q]); energies: also E_j = sum_{q
-  // in x} (P_j[q][q] + phi_j(q) / 2) per warp into sSum, doubled.
+  // Delta E of the state in sX from scratch: with phi_j(q) = sum_{r in x}
+  // P_j[r][q], Delta E_j(q) = P_j[q][q] + phi_j(q), or -phi_j(q) where x_q = 1;
+  // energies: also E_j = sum_{q in x} (P_j[q][q] + phi_j(q)) / 2 per warp into
+  // sSum, doubled.  Rows of P come from L2, one for each set bit, so a worker
+  // reads those of kRows bits for all of its words at once.  (Word after word,
+  // one row at a time: 361 ms for 16 replicas of m = 200 with two objectives
+  // whose 6,000 iterations mostly rebuild, 45 like this; 600 of m = 700 with
+  // three 3,023 and 550; 64 of m = 300 with three in 64 bits 677 and 136.)
+  constexpr int kRows = K * N <= 8 ? 4 : K * N <= 16 ? 2 : 1;
   auto rebuild = [&](bool energies) {
     __syncthreads();  // sX is complete
-    int64_t part[K];
-#pragma unroll
-    for (int j = 0; j < K; ++j) part[j] = 0;
     xn = 0u;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-      const int q = bit_of(k);
-      const bool in = q < m;
-      const uint32_t xq = w0 + k < W ? (sX[w0 + k] >> lane) & 1u : 0u;
-      xn |= xq << k;
-      int64_t phi[K];
+      if (w0 + k < W) xn |= ((sX[w0 + k] >> lane) & 1u) << k;
 #pragma unroll
-      for (int j = 0; j < K; ++j) phi[j] = 0;
-      if (w0 + k < W)
-        for (int w = 0; w < W; ++w) {
-          uint32_t word = uni(sX[w]);
-          while (word) {
-            const int r = w * 32 + __ffs(word) - 1;
-            word &= word - 1u;
-            if (in && r != q) {
+      for (int j = 0; j < K; ++j) dE[j][k] = 0;
+    }
+    const int32_t *own[K];  // the lane's first entry of row 0 (entries past m count for nobody)
 #pragma unroll
-              for (int j = 0; j < K; ++j) phi[j] += A.P[j * mm + (size_t)r * m + q];
-            }
-          }
+    for (int j = 0; j < K; ++j) own[j] = A.P + j * mm + 32 * w0 + lane;
+    for (int w = 0; wid < G && w < W; ++w) {
+      uint32_t word = uni(sX[w]);
+      while (word) {
+        int32_t pv[kRows][K][N];
+#pragma unroll
+        for (int u = 0; u < kRows; ++u) {
+          // (row 0 for nobody past the word's last bit: a mask and not a test,
+          // which would keep the rows' loads apart)
+          const int32_t some = word != 0u ? -1 : 0;
+          const int at = (some ? 32 * w + __ffs(word) - 1 : 0) * m;
+          word &= word - 1u;
+#pragma unroll
+          for (int j = 0; j < K; ++j)
+#pragma unroll
+            for (int k = 0; k < N; ++k) pv[u][j][k] = __ldg(own[j] + at + 32 * k) & some;
         }
 #pragma unroll
+        for (int u = 0; u < kRows; ++u)
+#pragma unroll
+          for (int k = 0; k < N; ++k)
+#pragma unroll
+            for (int j = 0; j < K; ++j) dE[j][k] += pv[u][j][k];
+      }
+    }
+    int64_t part[K];
+#pragma unroll
+    for (int j = 0; j < K; ++j) part[j] = 0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const int q = bit_of(k);
+      const bool in = q < m, xq = (xn >> k) & 1u;
+#pragma unroll
       for (int j = 0; j < K; ++j) {
-        const int64_t d = in ? A.P[j * mm + (size_t)q * m + q] : 0;
+        const int32_t d = in ? A.P[j * mm + (size_t)q * m + q] : 0;
+        if (xq) part[j] += (int64_t)d + dE[j][k];
         // (past m: a value no trial accepts)
-        dE[j][k] = in ? (dE_t)(xq ? -(d + phi[j]) : d + phi[j]) : (dE_t)0x3FFFFFFF;
-        if (xq) part[j] += 2 * d + phi[j];
+        dE[j][k] = !in ? (dE_t)0x3FFFFFFF : xq ? -dE[j][k] : d + dE[j][k];
       }
     }
     if (energies) {
@@ -910,7 +933,7 @@ moda_status moda_qubo_create(int32_t K, int32_t m, const int32_t *Q, moda_qubo *
   if (K < 1 || K > kMaxK) return qfail(MODA_EINVAL, "K must be in [1, 3]");
   if (m < 1 || m > kMaxQBits) return qfail(MODA_EINVAL, "m must be in [1, 4096]");
   const size_t mm = (size_t)m * m;
-  std::vector<int32_t> P((size_t)K * mm);
+  std::vector<int32_t> P((size_t)K * mm + moda::kQPad, 0);
   for (int j = 0; j < K; ++j) {
     const int32_t *Qj = Q + (size_t)j * mm;
     for (int p = 0; p < m; ++p)

@@ -65,3 +65,21 @@ def test_shared_archive_scan(m, arc):
         c = int(res["count"][r])
         assert np.array_equal(res["E"][r, :c], orc["E"][r, :c])
         assert np.array_equal(moda.unpack_bits(res["bits"][r, :c], m), orc["bits"][r, :c])
+
+
+@pytest.mark.parametrize("K,m,mag", [(1, 96, 50), (2, 200, 50), (3, 130, 50), (1, 257, 2 ** 29),
+                                     (3, 70, 2 ** 29), (2, 2850, 8)])
+def test_rebuilds_of_landings(K, m, mag):
+    """Records off at a temperature at which most jumps land on members that may
+    accept: Delta E from the rows of the set bits, one to four at a time, words
+    with a ragged number of them."""
+    from paper_2205_13399_gb300 import moda
+    rng = np.random.default_rng(7 * m + K)
+    Q = np.triu(rng.integers(-mag, mag, (K, m, m)).astype(np.int32))
+    kw = dict(replicas=2, I_max=400 if m < 1000 else 120, seed=m, delta0=100.0 * mag * K,
+              deltaf=mag * 1.5, xi=0.03 if m < 1000 else 0.1)
+    res = moda.Qubo(Q).anneal(trace=True, field_cache="off", **kw).wait().read(trace=True)
+    orc = oracle.kqubo_run(oracle.KQubo(Q), trace=True, **kw)
+    assert np.array_equal(res["trace"], orc["trace"])
+    assert np.array_equal(moda.unpack_bits(res["x"], m), orc["x"])
+    assert np.array_equal(res["stats"], orc["stats"])
