@@ -362,8 +362,8 @@ __global__ void __maxnreg__(N == 4 ? 80 : 96) qubo_kernel(const QArgs A) {
       }
     };
     uint32_t t = 1;
-    if (I_max >= 1) trial(1);
     while (t <= I_max) {
+      trial(t);  // (its only place: the kernel's three roles share the instruction cache)
       const uint32_t sel = ring[t % kQRing].sel;
       __syncthreads();  // A(t)
       const uint32_t c = (uint32_t)count_of(t);
@@ -379,7 +379,6 @@ __global__ void __maxnreg__(N == 4 ? 80 : 96) qubo_kernel(const QArgs A) {
           break;
         }
         ++t;
-        trial(t);
         continue;
       }
       if (total == 0) {
@@ -392,22 +391,24 @@ __global__ void __maxnreg__(N == 4 ? 80 : 96) qubo_kernel(const QArgs A) {
         if (mode == kQEnd || mode == kQStayEnd) break;
         if (mode == kQLoad) {
           if (gR != nullptr) {
+            // (the record, while the store warp fetches the member's state)
             const dE_t *from = gR + (size_t)uni((int)sJ[3]) * K * m;
-            __syncthreads();  // sX is complete
-            xn = 0u;
 #pragma unroll
             for (int k = 0; k < N; ++k) {
               const int q = bit_of(k);
-              if (w0 + k < W) xn |= ((sX[w0 + k] >> lane) & 1u) << k;
 #pragma unroll
               for (int j = 0; j < K; ++j)
                 dE[j][k] = q < m ? from[(size_t)j * m + q] : (dE_t)0x3FFFFFFF;
             }
+            __syncthreads();  // sX is complete
+            xn = 0u;
+#pragma unroll
+            for (int k = 0; k < N; ++k)
+              if (w0 + k < W) xn |= ((sX[w0 + k] >> lane) & 1u) << k;
           } else {
             rebuild(false);
           }
         }
-        trial(t);
         continue;
       }
       // ---- one accepted bit at random (R11): rank r in ascending bit
@@ -477,7 +478,6 @@ __global__ void __maxnreg__(N == 4 ? 80 : 96) qubo_kernel(const QArgs A) {
       ++nflip;
       fresh = true;
       ++t;
-      trial(t);
     }
     return;
   }
