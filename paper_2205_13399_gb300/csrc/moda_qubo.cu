@@ -492,8 +492,7 @@ __global__ void __maxnreg__(N == 4 ? 80 : 96) qubo_kernel(const QArgs A) {
         for (int q = lane; q < W; q += 32) gB[(size_t)target * W + q] = sX[q];
       __syncwarp();
     };
-    auto refill = [&](uint32_t from, uint32_t t) {  // the ring holds t .. t + 47 at least
-      filled = ring_skip(filled, from, t);
+    auto refill = [&](uint32_t t) {  // the ring holds t .. t + 47 at least
       while (ring_short(filled, t)) {
         fill(filled + 1u);
         filled += 32u;
@@ -515,7 +514,7 @@ __global__ void __maxnreg__(N == 4 ? 80 : 96) qubo_kernel(const QArgs A) {
           if (p1) store(t);
           break;
         }
-        refill(t, t + 2u);
+        refill(t + 2u);
         ++t;
         continue;
       }
@@ -525,12 +524,12 @@ __global__ void __maxnreg__(N == 4 ? 80 : 96) qubo_kernel(const QArgs A) {
       __syncthreads();
       const uint32_t mode = uni(sJ[0]);
       const int slot = uni((int)sJ[2]);
-      const uint32_t from = t;
+      filled = ring_skip(filled, t, uni(sJ[1]));
       t = uni(sJ[1]);
       if (mode == kQEnd || mode == kQLoad)  // the member the jumps ended on (written here)
         for (int q = lane; q < W; q += 32) sX[q] = gB[(size_t)slot * W + q];
       if (mode == kQEnd || mode == kQStayEnd) break;
-      refill(from, t);
+      refill(t);
       if (mode == kQLoad) {
         if (gR != nullptr) __syncthreads();
         else rebuild(false);

@@ -1024,8 +1024,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       }
       __syncwarp();
     };
-    auto refill = [&](uint32_t from, uint32_t t) {  // the ring holds t .. t + 47 at least
-      filled = ring_skip(filled, from, t);
+    auto refill = [&](uint32_t t) {  // the ring holds t .. t + 47 at least
       while (ring_short(filled, t)) {
         fill(filled + 1u);
         filled += 32u;
@@ -1051,7 +1050,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
           if (EXT) snapshots(t);
           break;
         }
-        refill(t, t + 2u);
+        refill(t + 2u);
         ++t;
         continue;
       }
@@ -1061,14 +1060,14 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       __syncthreads();
       const uint32_t mode = uni(sJ[0]);
       const int slot = uni((int)sJ[2]);
-      const uint32_t from = t;
+      filled = ring_skip(filled, t, uni(sJ[1]));
       t = uni(sJ[1]);
       if (EXT) snapshots(mode == kRegEnd || mode == kRegStayEnd ? I_max : t - 1u);
       if (mode == kRegEnd || mode == kRegRebuild)  // the member the jumps ended on
         for (int q = lane; q < W; q += 32) sX[q] = gB[(size_t)slot * W + q];  // (written here)
       if (mode == kRegEnd || mode == kRegStayEnd) break;
-      if (mode == kRegRebuild) rebuild(false, [&] { refill(from, t); });
-      else refill(from, t);
+      if (mode == kRegRebuild) rebuild(false, [&] { refill(t); });
+      else refill(t);
       if (D > 0) __syncthreads();  // draws
     }
     __syncwarp();
