@@ -176,8 +176,9 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   RFlip *const sFlip = reinterpret_cast<RFlip *>(smem + SL.flip);      // [4]
   int32_t *const sTgt = reinterpret_cast<int32_t *>(smem + SL.tgt);    // [4] slot of the flip
   uint32_t *const sJ = reinterpret_cast<uint32_t *>(smem + SL.jump);   // jump: mode, t, slot
-  int32_t *const sHm = reinterpret_cast<int32_t *>(sJ + 4);  // WIDE: largest R_i + C_u, lagging
-  uint32_t *const sFlags = sJ + 5;  // rebuild: 1 a row with two bits, 2 one with more
+  // WIDE: largest R_i + C_u, lagging, for the trials of either parity
+  int32_t *const sHm = reinterpret_cast<int32_t *>(sJ + 4);
+  uint32_t *const sFlags = sJ + 6;  // rebuild: 1 a row with two bits, 2 one with more
   int32_t *const sR = reinterpret_cast<int32_t *>(smem + SL.rc);       // row counts
   int32_t *const sC = sR + kMaxN;                                      // column counts
   unsigned char *const sV = smem + SL.v2;                              // [n][2] bits of a row
@@ -355,7 +356,18 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     return (lenient ? fminf(f1, f2) : f1 + f2) + 0.f;
   };
   const bool wfloat = w1l < (INT64_C(1) << 31) && w2l < (INT64_C(1) << 31);
-  auto bits_hm = [&]() {  // WIDE: largest R_i + C_u (one warp)
+  // WIDE: largest R_i + C_u (the store warp).  Trial t + 1 reads what that warp
+  // published between the barriers A(t - 1) and A(t), three flips behind the
+  // trial's state, so which warp is faster decides nothing: not the form of the
+  // trial, nor the least penalty it reports, nor the counters that hang on it.
+  int hm = 0;
+  auto put_hm = [&](int par) {  // (both parities: -1)
+    if (WIDE && lane == 0) {
+      if (par != 1) sHm[0] = hm;
+      if (par != 0) sHm[1] = hm;
+    }
+  };
+  auto bits_hm = [&]() {
     int a = 0, b = 0;
     for (int i = lane; i < n; i += 32) {
       a = max(a, sR[i]);
@@ -363,7 +375,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     }
     a = __reduce_max_sync(kFull, a);
     b = __reduce_max_sync(kFull, b);
-    if (lane == 0) *sHm = a + b;
+    hm = a + b;
   };
 
   if (use_mma == 2) {
@@ -629,7 +641,10 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
         sSum[2 * wid + 1] = t2;
       }
     }
-    if (WIDE && wid == warps - 1) bits_hm();
+    if (WIDE && wid == warps - 1) {
+      bits_hm();
+      put_hm(-1);
+    }
     __syncthreads();
   };
 
@@ -713,7 +728,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       const float margin = EXT ? r.margin + 1e-6f * off : r.margin;
       // every |Delta E_k| of the state fits int32 (a bound on the counts that
       // lags by at most three flips, which the limit allows for)
-      const bool nar = !WIDE || uni(*reinterpret_cast<volatile int32_t *>(sHm)) <= hm_limit;
+      const bool nar = !WIDE || uni(sHm[t & 1u]) <= hm_limit;
       uint32_t a[K];  // penalties; floats where not nar
       float near = 3.0e38f;
       accb = 0u;
@@ -1037,6 +1052,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       __syncthreads();  // A(t)
       const int total = __reduce_add_sync(kFull, count_of(t));
       if (p2) store(t - 2u);
+      put_hm((int)(t & 1u));
       if (EXT && t > 2u) snapshots(t - 2u);
       if (total > 0 || by_offset) {
         p2 = p1;
@@ -1057,6 +1073,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       __syncthreads();
       if (p1) store(t - 1u);
       p1 = p2 = false;
+      put_hm(-1);
       __syncthreads();
       const uint32_t mode = uni(sJ[0]);
       const int slot = uni((int)sJ[2]);
