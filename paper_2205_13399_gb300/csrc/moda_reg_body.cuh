@@ -70,7 +70,8 @@ struct RRing {
   float margin;     // half width of the band the FP32 test leaves undecided
   uint32_t sel;     // select draw
   uint32_t hi;      // floor(delta T_max), at most 2^32 - 1
-  uint32_t pad[2];
+  int32_t hm;       // WIDE: largest R_i + C_u of the state tried, lagging
+  uint32_t pad;
 };
 static_assert(sizeof(RRing) == 32, "ring entry layout");
 
@@ -176,9 +177,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   RFlip *const sFlip = reinterpret_cast<RFlip *>(smem + SL.flip);      // [4]
   int32_t *const sTgt = reinterpret_cast<int32_t *>(smem + SL.tgt);    // [4] slot of the flip
   uint32_t *const sJ = reinterpret_cast<uint32_t *>(smem + SL.jump);   // jump: mode, t, slot
-  // WIDE: largest R_i + C_u, lagging, for the trials of either parity
-  int32_t *const sHm = reinterpret_cast<int32_t *>(sJ + 4);
-  uint32_t *const sFlags = sJ + 6;  // rebuild: 1 a row with two bits, 2 one with more
+  uint32_t *const sFlags = sJ + 4;  // rebuild: 1 a row with two bits, 2 one with more
   int32_t *const sR = reinterpret_cast<int32_t *>(smem + SL.rc);       // row counts
   int32_t *const sC = sR + kMaxN;                                      // column counts
   unsigned char *const sV = smem + SL.v2;                              // [n][2] bits of a row
@@ -225,7 +224,8 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     uint32_t c[4] = {0u, q, rep, kTagSelect};
     philox10(c, k0, k1);
     e.sel = c[0];
-    e.pad[0] = e.pad[1] = 0u;
+    e.hm = 0;
+    e.pad = 0u;
     ring[q % kRegRing] = e;
   };
   uint32_t filled = 64;
@@ -356,18 +356,12 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     return (lenient ? fminf(f1, f2) : f1 + f2) + 0.f;
   };
   const bool wfloat = w1l < (INT64_C(1) << 31) && w2l < (INT64_C(1) << 31);
-  // WIDE: largest R_i + C_u (the store warp).  Trial t + 1 reads what that warp
-  // published between the barriers A(t - 1) and A(t), three flips behind the
-  // trial's state, so which warp is faster decides nothing: not the form of the
-  // trial, nor the least penalty it reports, nor the counters that hang on it.
-  int hm = 0;
-  auto put_hm = [&](int par) {  // (both parities: -1)
-    if (WIDE && lane == 0) {
-      if (par != 1) sHm[0] = hm;
-      if (par != 0) sHm[1] = hm;
-    }
-  };
-  auto bits_hm = [&]() {
+  // WIDE: largest R_i + C_u (the store warp).  It goes into the ring entry of
+  // the trial it is for, before the barrier that trial follows: the entry of t +
+  // 2 between A(t) and A(t + 1), three flips behind that trial's state.  Which
+  // warp is faster then decides neither the form of a trial nor the least
+  // penalty it reports, nor the counters that hang on it.
+  auto bits_hm = [&]() -> int {
     int a = 0, b = 0;
     for (int i = lane; i < n; i += 32) {
       a = max(a, sR[i]);
@@ -375,7 +369,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     }
     a = __reduce_max_sync(kFull, a);
     b = __reduce_max_sync(kFull, b);
-    hm = a + b;
+    return a + b;
   };
 
   if (use_mma == 2) {
@@ -408,9 +402,9 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   // rows have at most two bits, else from blocks of rows of M in shared
   // memory.  Starts with a block barrier after which sX must be complete and
   // ends on one.  energies: also sums over the set bits of L_1 and L_2
-  // (2 c_k) per warp into sSum.  aside(): what the last (store) warp does while
+  // (2 c_k) per warp into sSum.  at: the iteration to be tried next.  aside(): what the last (store) warp does while
   // the others scatter the set bits and form M.
-  auto rebuild = [&](bool energies, auto &&aside) {
+  auto rebuild = [&](bool energies, uint32_t at, auto &&aside) {
     const bool helps = wid != warps - 1;
     for (int i = threadIdx.x; i < 2 * kMaxN; i += threads) sR[i] = 0;
     for (int i = threadIdx.x; i < kMaxN / 2; i += threads)
@@ -642,8 +636,8 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       }
     }
     if (WIDE && wid == warps - 1) {
-      bits_hm();
-      put_hm(-1);
+      const int hm = bits_hm();
+      if (lane < 2) ring[(at + (uint32_t)lane) % kRegRing].hm = hm;
     }
     __syncthreads();
   };
@@ -671,7 +665,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
   };
 
   __syncthreads();
-  rebuild(true, [] {});
+  rebuild(true, 1u, [] {});
 
   if (wid >= G && wid < G + D) {
     // ================= draw warps =================
@@ -696,7 +690,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
         const uint32_t mode = uni(sJ[0]);
         t = uni(sJ[1]);
         if (mode == kRegEnd || mode == kRegStayEnd) break;
-        if (mode == kRegRebuild) rebuild(false, [] {});
+        if (mode == kRegRebuild) rebuild(false, t, [] {});
         draw(t);
         draw(t + 1u);
         __syncthreads();
@@ -728,7 +722,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       const float margin = EXT ? r.margin + 1e-6f * off : r.margin;
       // every |Delta E_k| of the state fits int32 (a bound on the counts that
       // lags by at most three flips, which the limit allows for)
-      const bool nar = !WIDE || uni(sHm[t & 1u]) <= hm_limit;
+      const bool nar = !WIDE || uni(r.hm) <= hm_limit;
       uint32_t a[K];  // penalties; floats where not nar
       float near = 3.0e38f;
       accb = 0u;
@@ -894,7 +888,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
         const uint32_t mode = uni(sJ[0]);
         t = uni(sJ[1]);
         if (mode == kRegEnd || mode == kRegStayEnd) break;
-        if (mode == kRegRebuild) rebuild(false, [] {});
+        if (mode == kRegRebuild) rebuild(false, t, [] {});
         if (D > 0) __syncthreads();  // draws
         trial(t);
         continue;
@@ -1035,7 +1029,8 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
           sC[fu] += sgn;
         }
         __syncwarp();
-        bits_hm();
+        const int hm = bits_hm();
+        if (lane == 0) ring[(tp + 4u) % kRegRing].hm = hm;
       }
       __syncwarp();
     };
@@ -1051,8 +1046,8 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     while (t <= I_max) {
       __syncthreads();  // A(t)
       const int total = __reduce_add_sync(kFull, count_of(t));
-      if (p2) store(t - 2u);
-      put_hm((int)(t & 1u));
+      if (p2) store(t - 2u);  // (with the bound of trial t + 2)
+      else if (WIDE && lane == 0) ring[(t + 2u) % kRegRing].hm = ring[(t + 1u) % kRegRing].hm;
       if (EXT && t > 2u) snapshots(t - 2u);
       if (total > 0 || by_offset) {
         p2 = p1;
@@ -1073,7 +1068,6 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       __syncthreads();
       if (p1) store(t - 1u);
       p1 = p2 = false;
-      put_hm(-1);
       __syncthreads();
       const uint32_t mode = uni(sJ[0]);
       const int slot = uni((int)sJ[2]);
@@ -1083,7 +1077,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
       if (mode == kRegEnd || mode == kRegRebuild)  // the member the jumps ended on
         for (int q = lane; q < W; q += 32) sX[q] = gB[(size_t)slot * W + q];  // (written here)
       if (mode == kRegEnd || mode == kRegStayEnd) break;
-      if (mode == kRegRebuild) rebuild(false, [&] { refill(t); });
+      if (mode == kRegRebuild) rebuild(false, t, [&] { refill(t); });
       else refill(t);
       if (D > 0) __syncthreads();  // draws
     }
@@ -1363,7 +1357,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     __syncthreads();
     if (end) break;
     ++nrebuild;
-    rebuild(false, [] {});
+    rebuild(false, t, [] {});
     if (D > 0) __syncthreads();  // draws
   }
 
