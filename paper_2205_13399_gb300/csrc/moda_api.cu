@@ -1504,6 +1504,11 @@ cudaError_t read_wait(cudaStream_t st, bool *done) {
   return e == cudaErrorNotReady ? cudaSuccess : e;
 }
 
+// Reads through the host: up to this many members in all (16 replicas of n = 8
+// have 160; 128 of n = 25 about 13,000), and of one archive up to this many words
+// of states in one copy (2 MiB).
+constexpr size_t kFewMembers = 512, kSpanWords = size_t(1) << 19;
+
 // The non-dominated members of replica `rep` (or all, rep == -1) of an
 // archive held on the device as counts[q * ns + j], energies at
 // E + (q * ns + j) * s * 2 and states at bits + (q * ns + j) * s * W: the
@@ -1531,7 +1536,10 @@ moda_status archive_front(moda_run r, int32_t rep, moda_point *pts, int32_t cap,
   };
   bool have = false;
   const size_t head = 16;
-  if (most > 0) MODA_CUDA(list.get(head + most * sizeof(moda::FrontPoint), st, &have));
+  // few members: their energies are copied and sorted sooner than a kernel is
+  // launched and waited for
+  if (most > kFewMembers)
+    MODA_CUDA(list.get(head + most * sizeof(moda::FrontPoint), st, &have));
   if (have) {  // each replica's own front, behind a counter
     auto *total = static_cast<uint32_t *>(list.p);
     auto *out = reinterpret_cast<moda::FrontPoint *>(static_cast<unsigned char *>(list.p) + head);
@@ -1541,14 +1549,21 @@ moda_status archive_front(moda_run r, int32_t rep, moda_point *pts, int32_t cap,
     MODA_CUDA(read_wait(st, &have));
   }
   if (have) {
+    // the counter and the points that most fronts have, then the others
     const auto *out = static_cast<const unsigned char *>(list.p);
+    constexpr size_t point = sizeof(moda::FrontPoint);
+    const size_t guess = std::min<size_t>(most, 1024);
+    std::vector<unsigned char> begin(head + point * guess);
+    MODA_CUDA(fetch(begin.data(), out, begin.size()));
     uint32_t got = 0;
-    MODA_CUDA(fetch(&got, out, sizeof(got)));
+    memcpy(&got, begin.data(), sizeof(got));
     c.resize(got);
-    MODA_CUDA(fetch(c.data(), out + head, sizeof(moda::FrontPoint) * got));
+    memcpy(c.data(), begin.data() + head, point * std::min<size_t>(got, guess));
+    if (got > guess)
+      MODA_CUDA(fetch(c.data() + guess, out + head + point * guess, point * (got - guess)));
   }
-  const bool by_host = most > 0 && !have;
-  if (by_host) {  // every member, the archives of some replicas at a time
+  const bool late = list.p != nullptr && !have;  // kernels wait for room
+  if (most > 0 && !have) {  // every member, the archives of some replicas at a time
     const size_t longest = (size_t)std::min(*std::max_element(cnt.begin(), cnt.end()), s);
     const size_t row = 2 * sizeof(int64_t) * longest, pitch = 2 * sizeof(int64_t) * ns * s;
     const int rows =  // 16 MiB; one where the copy's pitch would pass its limit
@@ -1593,11 +1608,32 @@ moda_status archive_front(moda_run r, int32_t rep, moda_point *pts, int32_t cap,
   const size_t list_bytes = sizeof(moda::FrontPoint) * (size_t)wr;
   const size_t pb = moda::align_up(list_bytes, 16), state_bytes = sizeof(uint32_t) * state.size();
   have = false;
-  if (wr > 0 && !by_host) MODA_CUDA(words.get(pb + state_bytes, copies, &have));
-  if (have) {
+  if (wr > 0 && last - first == 1) {
+    // one archive: the slots from the first to the last of the front as they lie
+    int lo = s, hi = 0;
+    for (int k = 0; k < wr; ++k) {
+      lo = std::min(lo, keep[k].slot);
+      hi = std::max(hi, keep[k].slot);
+    }
+    const size_t span = (size_t)(hi - lo + 1) * W;
+    if (span <= kSpanWords) {
+      std::vector<uint32_t> all(span);
+      MODA_CUDA(fetch(all.data(), dbits + (((size_t)first * ns + j) * s + lo) * W,
+                      sizeof(uint32_t) * span));
+      for (int k = 0; k < wr; ++k)
+        std::copy_n(all.data() + (size_t)(keep[k].slot - lo) * W, W,
+                    state.data() + (size_t)k * W);
+      have = true;
+    }
+  }
+  const bool copied = have;
+  // (a list of up to 64 KiB is staged by the call and waits for nothing)
+  cudaStream_t up = list_bytes <= 65536 ? st : copies;
+  if (wr > 0 && !have && !late) MODA_CUDA(words.get(pb + state_bytes, up, &have));
+  if (have && !copied) {
     auto *out = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(words.p) + pb);
-    MODA_CUDA(cudaMemcpyAsync(words.p, keep.data(), list_bytes, cudaMemcpyHostToDevice, copies));
-    MODA_CUDA(cudaStreamSynchronize(copies));  // (the kernel runs on another stream)
+    MODA_CUDA(cudaMemcpyAsync(words.p, keep.data(), list_bytes, cudaMemcpyHostToDevice, up));
+    if (up != st) MODA_CUDA(cudaStreamSynchronize(up));
     MODA_CUDA(moda::launch_gather(dbits, static_cast<moda::FrontPoint *>(words.p), wr, s, (int)ns,
                                   (int)j, W, out, st));
     MODA_CUDA(read_wait(st, &have));
