@@ -1481,10 +1481,12 @@ struct ReadBuffer {
 
 // Waits for what was enqueued on `st`, but not long: the kernels of a read
 // wait for room on a device that runs are filling (up to the time one of their
-// blocks takes, 100 ms and more; front and gather take 20 us alone), and
-// reading through the host takes a few milliseconds.  False: not done.
+// blocks takes, 100 ms and more; front and gather take 20 us alone, 50 where
+// they fit beside the runs), and reading through the host takes a millisecond
+// or two.  (Beside 1,500 replicas of n = 40 5.9 ms a read with 1 ms here, 4.3
+// with 0.3.)  False: not done.
 cudaError_t read_wait(cudaStream_t st, bool *done) {
-  constexpr std::chrono::microseconds kReadWait(1000);
+  constexpr std::chrono::microseconds kReadWait(300);
   *done = false;
   cudaEvent_t ev = nullptr;
   cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
