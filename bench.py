@@ -232,6 +232,9 @@ def roofline_line(ops, seconds, sms, sm_max_mhz, per_unit):
     return {"bound": "alu", "achieved": achieved / 1e12, "peak": measured / 1e12,
             "unit": "Tops/s", "frac": achieved / measured, "traffic": None,
             "kernel": "anneal_kernel", "per_unit": per_unit,
+            "frac_is": "algorithmic work over the INT32 peak: every bit of every iteration "
+                       "counts, also of jumps settled by one compare, so it can pass 1 and is "
+                       "not the share of issue slots used",
             "peak_source": "measured: moda_probe_int_peak (INT32 lane-ops/s, all SMs)",
             "peak_derived": derived / 1e12,
             "smem_peak_GBps": smem / 1e9}

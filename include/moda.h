@@ -434,7 +434,7 @@ const char *moda_last_error(void);
  *   escape, replicas * s * r * ceil8(n^2) bytes <= 64 MiB (s = archive
  *   size; r = 8 when every |Delta E_k| of the instance stays below 2^31,
  *   i.e. B_k + w_k (2n + 1) < 2^31 with B_k the bound of moda_create_instance,
- *   else 16); the offset escape uses no scratch; at most 65,536 schedule
+ *   else 16); the offset escape is not limited by it; at most 65,536 schedule
  *   entries before delta reaches delta_f; params.trace = 0.
  *   params.field_cache and params.prefetch are ignored (the cache is used
  *   whenever the escape jumps to the archive).
