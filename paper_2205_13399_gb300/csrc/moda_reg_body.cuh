@@ -713,6 +713,14 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     // warp's words: accepted bits (ballots for a few words, else the lane's
     // own, word k at bit K - 1 - k), their count and the least penalty.
     constexpr bool BAL = K <= 4;
+    // Whether the trial stands at one place, the head of the loop, or at the end
+    // of each way through it.  Once is less code for the instruction cache that
+    // the roles share and spills less with many words (n = 100, 32 replicas
+    // 102.2 -> 95.2 ms, n = 76, 150 of them 84.7 -> 83.0, n = 50 48.6 -> 47.0, n = 60
+    // with snapshots 46.4 -> 45.5); with few, or beyond int32 with eight, the ends
+    // run on into the trial better (n = 41 beyond int32 61.5 against 65.7, n = 40
+    // normalised 29.1 and 30.5, n = 75 110.6 and 111.6).
+    constexpr bool ONCE = K >= 16 || (K == 8 && (!WIDE || EXT));
     uint32_t acc[BAL ? K : 1], accb = 0u, amin = 0u;
     int cnt = 0;
     int64_t Eoff = 0;  // the offset escape's E_off
@@ -858,11 +866,10 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
     };
 
     uint32_t t = 1;
-    if (I_max >= 1) {
-      if (D > 0) __syncthreads();
-      trial(1);
-    }
+    if (I_max >= 1 && D > 0) __syncthreads();
+    if (!ONCE && I_max >= 1) trial(1);
     while (t <= I_max) {
+      if (ONCE) trial(t);
       const uint32_t sel = ring[t % kRegRing].sel;
       __syncthreads();  // A(t): the trial's counts are complete
       const uint32_t c = (uint32_t)count_of(t);
@@ -879,7 +886,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
           break;
         }
         ++t;
-        trial(t);
+        if (!ONCE) trial(t);
         continue;
       }
       if (total == 0) {
@@ -890,7 +897,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
         if (mode == kRegEnd || mode == kRegStayEnd) break;
         if (mode == kRegRebuild) rebuild(false, t, [] {});
         if (D > 0) __syncthreads();  // draws
-        trial(t);
+        if (!ONCE) trial(t);
         continue;
       }
       // ---- one accepted bit at random (R11): rank r in ascending bit
@@ -982,7 +989,7 @@ __global__ void __maxnreg__(reg_regs(K)) reg_anneal_kernel(const RegLaunch L) {
           }
       }
       ++t;
-      trial(t);
+      if (!ONCE) trial(t);
     }
     return;
   }
